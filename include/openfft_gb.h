@@ -255,10 +255,11 @@ int openfft_decomp_degree(int Na, int Nb, int Nc, int P, int layout);
  * for this problem (see openfft_tuning_save below). */
 int openfft_set_tuning(openfft_plan_t plan, int mode, int candidate);
 
-/* Stage-kernel families: one warp per line (power-of-two lengths 32..512 and
- * the mixed-radix lengths 48..160), tiles of lines specialised per length, or
- * the generic kernel (any length); AUTO takes the first of these that exists
- * for the length. */
+/* Stage-kernel families: one warp per line (power-of-two lengths 32..512),
+ * tiles of lines specialised per length, or the generic kernel (any length);
+ * AUTO takes the warp kernel where it exists, for the other lengths (and not
+ * for NATIVE arithmetic) tiles with a radix plan chosen per length, else the
+ * tile or the generic kernel. */
 enum { OPENFFT_KERNEL_AUTO = 0, OPENFFT_KERNEL_WARP = 1, OPENFFT_KERNEL_TILE = 2, OPENFFT_KERNEL_GENERIC = 3 };
 
 /* Number of execution candidates of this plan and a description of one

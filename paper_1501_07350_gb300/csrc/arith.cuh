@@ -62,6 +62,8 @@ struct ArF32 {
     __device__ __forceinline__ static C mul(C a, W w) {
         return make_float2(fmaf(a.x, w.x, -a.y * w.y), fmaf(a.x, w.y, a.y * w.x));
     }
+    // multiply by the complex constant re + i im
+    __device__ __forceinline__ static C mulc(C a, double re, double im) { return mul(a, make_float2((float)re, (float)im)); }
     __device__ __forceinline__ static C scale(C a, double k) {
         const float kf = (float)k;
         return make_float2(a.x * kf, a.y * kf);
@@ -237,6 +239,99 @@ template <class A> struct Dft<A, 8> {
         x[1] = A::add(e[1], o1);   x[5] = A::sub(e[1], o1);
         x[2] = A::add(e[2], o2);   x[6] = A::sub(e[2], o2);
         x[3] = A::add(e[3], o3);   x[7] = A::sub(e[3], o3);
+    }
+};
+
+// Composite radices.  Coprime factors use the prime-factor index maps (input
+// n = (R2 n1 + R1 n2) mod R, output k = (e1 k1 + e2 k2) mod R with e1 = 1 mod R1,
+// 0 mod R2 and e2 the reverse): no twiddles between the two sub-transforms.
+template <class A, int R1, int R2, int E1, int E2>
+__device__ __forceinline__ void dft_coprime(typename A::C* x)
+{
+    constexpr int R = R1 * R2;
+    typename A::C y[R];
+#pragma unroll
+    for (int n1 = 0; n1 < R1; ++n1) {
+        typename A::C r[R2];
+#pragma unroll
+        for (int n2 = 0; n2 < R2; ++n2) r[n2] = x[(R2 * n1 + R1 * n2) % R];
+        Dft<A, R2>::run(r);
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) y[n1 * R2 + k2] = r[k2];
+    }
+#pragma unroll
+    for (int k2 = 0; k2 < R2; ++k2) {
+        typename A::C c[R1];
+#pragma unroll
+        for (int n1 = 0; n1 < R1; ++n1) c[n1] = y[n1 * R2 + k2];
+        Dft<A, R1>::run(c);
+#pragma unroll
+        for (int k1 = 0; k1 < R1; ++k1) x[(E1 * k1 + E2 * k2) % R] = c[k1];
+    }
+}
+template <class A> struct Dft<A, 6> { __device__ __forceinline__ static void run(typename A::C* x) { dft_coprime<A, 2, 3, 3, 4>(x); } };
+template <class A> struct Dft<A, 10> { __device__ __forceinline__ static void run(typename A::C* x) { dft_coprime<A, 2, 5, 5, 6>(x); } };
+template <class A> struct Dft<A, 12> { __device__ __forceinline__ static void run(typename A::C* x) { dft_coprime<A, 3, 4, 4, 9>(x); } };
+template <class A> struct Dft<A, 15> { __device__ __forceinline__ static void run(typename A::C* x) { dft_coprime<A, 3, 5, 10, 6>(x); } };
+
+// R = R1^2 (9, 16): rows, constant twiddles W_R^(n1 k2), columns.
+constexpr double kCos1_9 = 0.76604444311897803520239265055541668;    // cos / sin (2 pi k / 9), k = 1, 2, 4
+constexpr double kSin1_9 = 0.64278760968653932632264340990726343;
+constexpr double kCos2_9 = 0.17364817766693034885171662676931480;
+constexpr double kSin2_9 = 0.98480775301220805936674302458952301;
+constexpr double kCos4_9 = -0.93969262078590838405410927732473147;
+constexpr double kSin4_9 = 0.34202014332566873304409961468225958;
+constexpr double kCos1_16 = 0.92387953251128675612818318939678829;   // cos / sin (2 pi / 16)
+constexpr double kSin1_16 = 0.38268343236508977172845998403039887;
+
+template <class A> struct Dft<A, 9> {
+    __device__ __forceinline__ static void run(typename A::C* x) {
+        typename A::C y[9];
+#pragma unroll
+        for (int n1 = 0; n1 < 3; ++n1) {
+            typename A::C r[3] = {x[n1], x[n1 + 3], x[n1 + 6]};
+            Dft<A, 3>::run(r);
+            y[3 * n1] = r[0]; y[3 * n1 + 1] = r[1]; y[3 * n1 + 2] = r[2];
+        }
+        y[4] = A::mulc(y[4], kCos1_9, -kSin1_9);
+        y[5] = A::mulc(y[5], kCos2_9, -kSin2_9);
+        y[7] = A::mulc(y[7], kCos2_9, -kSin2_9);
+        y[8] = A::mulc(y[8], kCos4_9, -kSin4_9);
+#pragma unroll
+        for (int k2 = 0; k2 < 3; ++k2) {
+            typename A::C c[3] = {y[k2], y[3 + k2], y[6 + k2]};
+            Dft<A, 3>::run(c);
+            x[k2] = c[0]; x[k2 + 3] = c[1]; x[k2 + 6] = c[2];
+        }
+    }
+};
+
+template <class A> struct Dft<A, 16> {
+    __device__ __forceinline__ static void run(typename A::C* x) {
+        typename A::C y[16];
+#pragma unroll
+        for (int n1 = 0; n1 < 4; ++n1) {
+            typename A::C r[4] = {x[n1], x[n1 + 4], x[n1 + 8], x[n1 + 12]};
+            Dft<A, 4>::run(r);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) y[4 * n1 + k] = r[k];
+        }
+        y[5] = A::mulc(y[5], kCos1_16, -kSin1_16);
+        y[6] = A::mulc(y[6], kSqrtHalf, -kSqrtHalf);
+        y[7] = A::mulc(y[7], kSin1_16, -kCos1_16);
+        y[9] = A::mulc(y[9], kSqrtHalf, -kSqrtHalf);
+        y[10] = A::mul_mi(y[10]);
+        y[11] = A::mulc(y[11], -kSqrtHalf, -kSqrtHalf);
+        y[13] = A::mulc(y[13], kSin1_16, -kCos1_16);
+        y[14] = A::mulc(y[14], -kSqrtHalf, -kSqrtHalf);
+        y[15] = A::mulc(y[15], -kCos1_16, kSin1_16);
+#pragma unroll
+        for (int k2 = 0; k2 < 4; ++k2) {
+            typename A::C c[4] = {y[k2], y[4 + k2], y[8 + k2], y[12 + k2]};
+            Dft<A, 4>::run(c);
+#pragma unroll
+            for (int k1 = 0; k1 < 4; ++k1) x[k2 + 4 * k1] = c[k1];
+        }
     }
 };
 

@@ -109,7 +109,10 @@ struct ArDP {
     __device__ __forceinline__ static W warp_twiddle(const W* tw, int off, int m, int j, int k, int)
     {
         const int e = off + (j - 1) * m + k;
-        const float4 q = __ldg(reinterpret_cast<const float4*>(tw) + e);
+        return make_w(__ldg(reinterpret_cast<const float4*>(tw) + e));
+    }
+    __device__ __forceinline__ static W make_w(float4 q)
+    {
         const u64 xx = p2_splat(q.x), yy = p2_splat(q.y), zz = p2_splat(q.z), ww = p2_splat(q.w);
         W w;
         w.a.x = xx;

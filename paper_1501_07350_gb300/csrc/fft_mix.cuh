@@ -1,0 +1,238 @@
+// fft_mix.cuh -- FFT stage kernel for the line lengths that have no kernel
+// compiled for them alone: any n <= 2048 with factors 2, 3, 5 and 7, in the packed
+// double-float and the FP32 arithmetic.
+//
+// A CTA takes tiles of G lines.  The radix plan is chosen on the host per length
+// (mix_plan): few passes of large radices (composite ones up to 10 in
+// double-float, 16 in FP32, whose coprime factors need no twiddles between
+// them), each pass compiled per radix, strides and counts at run time.
+//
+// Tile layout in shared memory: [position][G lines], so the lanes of a warp take
+// consecutive lines at one position: every pass reads and writes rows of
+// G elements whatever the radix and the length, a twiddle is one broadcast load
+// for the G lines (from the CTA's own copy of the length's table), and the last pass's results leave for global memory straight
+// from registers, G consecutive elements per frequency (the transposed store) or
+// 32 / G consecutive frequencies per line (the contiguous one).  Rows of 128 bytes
+// are padded by one element, so that the copies in (lanes along a line) are free
+// of bank conflicts too; rows of 64 bytes are not, and their copies run with
+// lanes across the lines (two consecutive positions fill the banks).
+//
+// Passes alternate between two tile buffers, one barrier each.  The last pass reads
+// one buffer and writes global memory, so the next tile's copies (cp.async) go into
+// the other buffer while it runs.
+#pragma once
+#include "arith.cuh"
+#include "arith_pair.cuh"
+#include "fft_stage.h"
+#include "fft_tile.cuh"
+#include "stage_io.cuh"
+
+namespace ofg {
+
+constexpr int kMixMaxPasses = 11;
+
+struct MixPass {
+    int radix;
+    int nbf;                    // butterflies of one line: n / radix
+    int m;                      // product of the earlier radices
+    int s;                      // nbf / m: twiddle exponent step
+    uint32_t inv;               // ceil(2^20 / m): b / m = (b inv) >> 20 for b m < 2^20
+};
+struct MixPlan {
+    int npass;
+    int slots;                  // threads per line of a tile
+    MixPass pass[kMixMaxPasses];
+};
+
+// threads per CTA at most, and the CTAs of that size the registers are sized for
+constexpr int kMixMaxThreads = 512;
+constexpr int mix_min_ctas() { return 2; }
+
+// entry e of the tile's copy of the twiddle table
+__device__ __forceinline__ ArF32::W mix_twiddle(const ArF32::C* tw, int e) { return tw[e]; }
+__device__ __forceinline__ ArDP::W mix_twiddle(const ArDP::C* tw, int e)
+{
+    return ArDP::make_w(reinterpret_cast<const float4*>(tw)[e]);
+}
+
+// a complex128 element that was copied as the bits of a double-float one
+__device__ __forceinline__ ArDP::C c128_bits(ArDP::C x)
+{
+    return Io<ArDP>::from_c128(make_double2(__longlong_as_double((long long)x.x), __longlong_as_double((long long)x.y)));
+}
+
+template <class A, int G>
+struct Mix {
+    using C = typename A::C;
+    static constexpr int E = sizeof(C);
+    // lanes of a warp: lines fastest, or (line, slot parity) with the parity fastest
+    static constexpr bool kPairs = E * G != 128 || E == 8;
+    static constexpr int kUnits = 128 / E;                    // elements of one shared-memory wavefront
+
+    __host__ __device__ static int pitch(int n)
+    {
+        if (!kPairs) return n | 1;
+        return n + (2 - n % kUnits + kUnits) % kUnits;
+    }
+    __device__ __forceinline__ static int line_of(int tid) { return kPairs ? (tid >> 1) % G : tid % G; }
+    __device__ __forceinline__ static int slot_of(int tid) { return kPairs ? (tid & 1) + 2 * (tid / (2 * G)) : tid / G; }
+
+    // Copies of a tile: `valid` lines, lstride apart from line0 on, a warp per line
+    // in 16-byte pieces (8 bytes where an odd length leaves lines unaligned).
+    __device__ __forceinline__ static void issue_load(const StageArgs& p, int64_t line0, int64_t lstride, int valid, C* buf,
+                                                      int ld, int tid, int T)
+    {
+        const int n = p.n, lane = tid & 31;
+        for (int g = tid >> 5; g < valid; g += T >> 5) {
+            const int64_t e = (line0 + g * lstride) * n;
+            const char* src = reinterpret_cast<const char*>(p.in) + e * E;
+            C* dst = buf + g * ld;
+            if (E == 16 || (n & 1)) {
+#pragma unroll 4
+                for (int i = lane; i < n; i += 32)
+                    if (in_bounds(p.chk, e + i, p.in_elems)) cp_async<E>(dst + i, src + i * E);
+            } else {
+#pragma unroll 4
+                for (int i = 2 * lane; i < n; i += 64)
+                    if (in_bounds(p.chk, e + i, p.in_elems) && in_bounds(p.chk, e + i + 1, p.in_elems))
+                        cp_async<16>(dst + i, src + i * E);
+            }
+        }
+        cp_async_commit();
+    }
+
+    template <bool CONJ_SCALE, bool EXT, int R>
+    __device__ __forceinline__ static void store(const StageArgs& p, int64_t o, int64_t step, const C* v)
+    {
+        constexpr int EB = EXT ? Io<A>::kExtBytes : Io<A>::kMidBytes;
+        char* ptr = reinterpret_cast<char*>(p.out) + o * EB;
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            if (in_bounds(p.chk, o + q * step, p.out_elems)) put<A, CONJ_SCALE, EXT>(ptr, v[q], p.scale);
+            ptr += step * EB;
+        }
+    }
+
+    // One pass from buffer src to buffer dst, or, the last one, to global memory.
+    template <int R, bool FIRST>
+    __device__ __forceinline__ static void pass(const StageArgs& p, const MixPass& ps, bool last, const TileGeom& tg,
+                                                const C* src, C* dst, const C* tw, int g, int slot, int slots)
+    {
+        // src, dst: this thread's line
+        const int nbf = ps.nbf;
+        for (int b = slot; b < nbf; b += slots) {
+            C v[R];
+            const C* x = src + b;
+#pragma unroll
+            for (int j = 0; j < R; ++j) v[j] = x[j * nbf];
+            int pos = b * R;                               // of the first result: t m R + k, b = t m + k
+            if constexpr (FIRST) {
+                if constexpr (Io<A>::kConverts) {
+                    if (p.in_fmt == FMT_C128) {
+#pragma unroll
+                        for (int j = 0; j < R; ++j) v[j] = c128_bits(v[j]);
+                    }
+                }
+                if (p.conj_in) {
+#pragma unroll
+                    for (int j = 0; j < R; ++j) v[j] = A::conj(v[j]);
+                }
+            } else {
+                const int t = (int)(((uint32_t)b * ps.inv) >> 20), k = b - t * ps.m;
+                pos = t * ps.m * R + k;
+                const int ks = k * ps.s;
+#pragma unroll
+                for (int j = 1; j < R; ++j) v[j] = A::mul(v[j], mix_twiddle(tw, j * ks));
+            }
+            Dft<A, R>::run(v);
+            if (!last) {
+                C* y = dst + pos;
+#pragma unroll
+                for (int q = 0; q < R; ++q) y[q * ps.m] = v[q];
+            } else {
+                const int64_t o = tg.obase + g * tg.ostride + b * p.Sk, step = ps.m * p.Sk;
+                const bool ext = p.out_fmt != FMT_DF;
+                if (p.conj_out) {
+                    if (ext) store<true, true, R>(p, o, step, v);
+                    else store<true, false, R>(p, o, step, v);
+                } else {
+                    if (ext) store<false, true, R>(p, o, step, v);
+                    else store<false, false, R>(p, o, step, v);
+                }
+            }
+        }
+    }
+
+    template <bool FIRST>
+    __device__ __forceinline__ static void dispatch(const StageArgs& p, const MixPass& ps, bool last, const TileGeom& tg,
+                                                    const C* src, C* dst, const C* tw, int g, int slot, int slots)
+    {
+        switch (ps.radix) {
+        case 2: pass<2, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+        case 3: pass<3, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+        case 4: pass<4, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+        case 5: pass<5, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+        case 6: pass<6, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+        case 7: pass<7, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+        case 8: pass<8, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+        case 10: pass<10, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+        default:
+            if constexpr (E == 8) {
+                switch (ps.radix) {
+                case 9: pass<9, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+                case 12: pass<12, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+                case 15: pass<15, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+                default: pass<16, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+                }
+            }
+            break;
+        }
+    }
+};
+
+template <class A, int G>
+__global__ void __launch_bounds__(kMixMaxThreads, mix_min_ctas())
+fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t ntiles)
+{
+    using M = Mix<A, G>;
+    using C = typename A::C;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int ld = M::pitch(p.n);
+    C* cur = reinterpret_cast<C*>(smem_raw);
+    C* oth = cur + G * ld;
+    C* tw = oth + G * ld;
+    const int tid = threadIdx.x, T = blockDim.x;
+    const int g = M::line_of(tid), slot = M::slot_of(tid), slots = plan.slots, at = g * ld;
+    int64_t tile = blockIdx.x;
+    TileGeom tg = tile_geom(p, tile, G);                // the grid has at most ntiles CTAs
+    for (int i = tid; i < p.n; i += T) cp_async<M::E>(tw + i, reinterpret_cast<const C*>(p.tw) + i);
+    M::issue_load(p, tg.line0, tg.lstride, tg.valid, cur, ld, tid, T);
+    for (; tile < ntiles; tile += gridDim.x) {
+        const int64_t next = tile + gridDim.x;
+        const TileGeom tn = tile_geom(p, next < ntiles ? next : tile, G);
+        const bool mine = g < tg.valid;
+        cp_async_wait_all();
+        __syncthreads();
+        const int np = plan.npass;
+        if (np > 1) {
+            if (mine) M::template dispatch<true>(p, plan.pass[0], false, tg, cur + at, oth + at, tw, g, slot, slots);
+            __syncthreads();
+            for (int ps = 1; ps < np - 1; ++ps) {
+                C* t = cur; cur = oth; oth = t;
+                if (mine) M::template dispatch<false>(p, plan.pass[ps], false, tg, cur + at, oth + at, tw, g, slot, slots);
+                __syncthreads();
+            }
+            // every thread has read `cur`: it takes the next tile while the last pass runs
+            if (next < ntiles) M::issue_load(p, tn.line0, tn.lstride, tn.valid, cur, ld, tid, T);
+            if (mine) M::template dispatch<false>(p, plan.pass[np - 1], true, tg, oth + at, cur + at, tw, g, slot, slots);
+        } else {
+            if (next < ntiles) M::issue_load(p, tn.line0, tn.lstride, tn.valid, oth, ld, tid, T);
+            if (mine) M::template dispatch<true>(p, plan.pass[0], true, tg, cur + at, oth + at, tw, g, slot, slots);
+            C* t = cur; cur = oth; oth = t;
+        }
+        tg = tn;
+    }
+    cp_async_wait_all();
+}
+
+}  // namespace ofg

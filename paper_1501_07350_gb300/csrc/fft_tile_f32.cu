@@ -18,8 +18,8 @@ cudaError_t launch_tile_f32(const StageLaunch& L, cudaStream_t st, bool* handled
         cudaError_t e = L.args.G == 8 ? launch_warp_g<ArF32, 8>(L, st, handled) : launch_warp_g<ArF32, 16>(L, st, handled);
         if (*handled || e) return e;
     }
-    if ((L.family == KERNEL_AUTO || L.family == KERNEL_WARP) && warp_mixed_length(L.args.n)) {
-        cudaError_t e = launch_warp_mixed_f32(L, st, handled);
+    if (L.family == KERNEL_AUTO) {
+        cudaError_t e = launch_mix_f32(L, st, handled);
         if (*handled || e) return e;
     }
     if (L.family == KERNEL_WARP) return cudaSuccess;
