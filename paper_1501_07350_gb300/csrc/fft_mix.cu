@@ -128,8 +128,7 @@ cudaError_t launch_mix_g(const StageLaunch& L, cudaStream_t st, bool* handled)
     a.ngroups = (Mg + G - 1) / G;
     const int64_t ntiles = a.ngroups * (a.group_i2 ? a.M1 : a.M2);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)L.sms * ml.per_sm, ntiles));
-    kern<<<(unsigned)grid, ml.threads, ml.smem, st>>>(a, ml.plan, ntiles);
-    return cudaGetLastError();
+    return launch_chained(kern, (unsigned)grid, ml.threads, ml.smem, st, a, ml.plan, ntiles);
 }
 
 }  // namespace

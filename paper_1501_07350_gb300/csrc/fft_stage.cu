@@ -41,6 +41,8 @@ fft_stage_kernel(const StageArgs p)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int64_t s_in[kMaxLinesPerCta];
     __shared__ int64_t s_out[kMaxLinesPerCta];
+    grid_wait();
+    grid_release();
     generic_stage_tile<A>(p, blockIdx.x, smem_raw, s_in, s_out);
 }
 
@@ -172,11 +174,10 @@ cudaError_t launch_stage(const StageLaunch& L0, cudaStream_t st)
     }
     const unsigned grid = (unsigned)L.grid;
     switch (L.arith) {
-    case ARITH_F64: fft_stage_kernel<ArF64><<<grid, kStageThreads, L.smem, st>>>(L.args); break;
-    case ARITH_F32: fft_stage_kernel<ArF32><<<grid, kStageThreads, L.smem, st>>>(L.args); break;
-    default: fft_stage_kernel<ArDF><<<grid, kStageThreads, L.smem, st>>>(L.args); break;
+    case ARITH_F64: return launch_chained(fft_stage_kernel<ArF64>, grid, kStageThreads, L.smem, st, L.args);
+    case ARITH_F32: return launch_chained(fft_stage_kernel<ArF32>, grid, kStageThreads, L.smem, st, L.args);
+    default: return launch_chained(fft_stage_kernel<ArDF>, grid, kStageThreads, L.smem, st, L.args);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_twiddles(int n, int fmt, void* out, cudaStream_t st)

@@ -62,6 +62,34 @@ enum { KERNEL_AUTO = 0, KERNEL_WARP = 1, KERNEL_TILE = 2, KERNEL_GENERIC = 3 };
 enum { KERNEL_R2C = 4, KERNEL_C2R = 5 };
 cudaError_t launch_real_stage(const StageLaunch& L, cudaStream_t st);
 
+// Stage kernels are launched with programmatic stream serialisation: a stage's CTAs
+// may become resident while the stage before it drains, and wait there
+// (grid_wait, which every stage kernel passes before it touches global memory)
+// until that grid has completed and its writes are visible.  It takes the launch
+// gap, about 2 us, out of the chain of stages: 32^3 complex128 went from 16.4 to
+// 11.8 us a transform.  A CTA lets the next stage start (grid_release) only when
+// it begins its last tile: released at its start, the next stage's CTAs gathered on
+// the SMs that had room first, and 240x288x320 complex64 took 316 us instead of 227.
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... Args>
+cudaError_t launch_chained(void (*kern)(P...), unsigned grid, int threads, size_t smem, cudaStream_t st, const Args&... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+#endif
+
 cudaError_t stage_kernels_init(int max_dyn_smem);
 // Device allocation of the library's workspaces (capi.cu): cudaMalloc, except
 // that a test control (openfft_debug_alloc_fail) can make the n-th call fail

@@ -278,11 +278,13 @@ fft_tile_kernel(const StageArgs p, int64_t ntiles)
     const int g_mine = tid % G, slot = tid / G;
     const typename A::W* tw = reinterpret_cast<const typename A::W*>(p.tw);
     const bool convert = Io<A>::kConverts && p.in_fmt == FMT_C128;
+    grid_wait();
 
     int64_t tile = blockIdx.x;
     if (tile < ntiles) tile_issue_loads<A, N, G, T>(p, tile_geom(p, tile, G), cur, tid);
     for (; tile < ntiles; tile += gridDim.x) {
         const TileGeom tg = tile_geom(p, tile, G);
+        if (tile + gridDim.x >= ntiles) grid_release();
         cp_async_wait_all();
         if (convert) { if (p.conj_in) tile_fix<A, N, G, T, true, true>(cur, tid); else tile_fix<A, N, G, T, true, false>(cur, tid); }
         else if (p.conj_in) tile_fix<A, N, G, T, false, true>(cur, tid);
@@ -327,8 +329,7 @@ cudaError_t launch_tile_n(const StageLaunch& L, cudaStream_t st)
     int64_t grid = (int64_t)L.sms * blocks_per_sm;
     if (grid > ntiles) grid = ntiles;
     if (grid < 1) grid = 1;
-    fft_tile_kernel<A, N, G, T><<<(unsigned)grid, T, smem, st>>>(L.args, ntiles);
-    return cudaGetLastError();
+    return launch_chained(fft_tile_kernel<A, N, G, T>, (unsigned)grid, T, smem, st, L.args, ntiles);
 }
 
 // Launch the specialised kernel for (N, G) if there is one; *handled = false otherwise.

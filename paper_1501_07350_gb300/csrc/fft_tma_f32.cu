@@ -54,6 +54,7 @@ fft_warp_tma_f32_kernel(const StageArgs p, int64_t ntiles, const __grid_constant
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g0 = warp * L;
     const A::W* tw = A::table(p.tw, N);
+    grid_wait();
 
     int64_t tile = blockIdx.x;
     if (tile < ntiles) {
@@ -62,6 +63,7 @@ fft_warp_tma_f32_kernel(const StageArgs p, int64_t ntiles, const __grid_constant
         for (int i = 0; i < L; ++i) warp_issue_load<A, N>(p, tg, g0 + i, cur + (g0 + i) * LS, lane);
     }
     for (; tile < ntiles; tile += gridDim.x) {
+        if (tile + gridDim.x >= ntiles) grid_release();
         C* line0 = cur + g0 * LS;
         cp_async_wait_all();
         if (p.conj_in) {
@@ -151,8 +153,7 @@ cudaError_t launch_f32_tma_n(const StageLaunch& L, cudaStream_t st, bool* handle
     int64_t grid = (int64_t)L.sms * per_sm;
     if (grid > ntiles) grid = ntiles;
     if (grid < 1) grid = 1;
-    kern<<<(unsigned)grid, f32_tma_threads<N, G>(), smem, st>>>(L.args, ntiles, map);
-    return cudaGetLastError();
+    return launch_chained(kern, (unsigned)grid, f32_tma_threads<N, G>(), smem, st, L.args, ntiles, map);
 }
 
 }  // namespace

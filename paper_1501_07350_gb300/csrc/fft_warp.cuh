@@ -274,6 +274,7 @@ fft_warp_kernel(const StageArgs p, int64_t ntiles)
     const int g0 = warp * L;                // this warp's first line of the tile
     const typename A::W* tw = A::table(p.tw, N);
     const bool convert = Io<A>::kConverts && p.in_fmt == FMT_C128;
+    grid_wait();
 
     int64_t tile = blockIdx.x;
     if (DB && tile < ntiles) {
@@ -283,6 +284,7 @@ fft_warp_kernel(const StageArgs p, int64_t ntiles)
     }
     for (; tile < ntiles; tile += gridDim.x) {
         const TileGeom tg = tile_geom(p, tile, G);
+        if (tile + gridDim.x >= ntiles) grid_release();
         C* line0 = cur + g0 * LS;
         if (!DB) {
 #pragma unroll
@@ -329,8 +331,7 @@ cudaError_t launch_warp_n(const StageLaunch& L, cudaStream_t st)
     int64_t grid = (int64_t)L.sms * blocks_per_sm;
     if (grid > ntiles) grid = ntiles;
     if (grid < 1) grid = 1;
-    fft_warp_kernel<A, N, G><<<(unsigned)grid, T, smem, st>>>(L.args, ntiles);
-    return cudaGetLastError();
+    return launch_chained(fft_warp_kernel<A, N, G>, (unsigned)grid, T, smem, st, L.args, ntiles);
 }
 
 // power-of-two lengths go to the warp-per-line kernel

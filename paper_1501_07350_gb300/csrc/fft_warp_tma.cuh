@@ -264,9 +264,11 @@ fft_warp_tma_kernel(const StageArgs p, int64_t ntiles, const __grid_constant__ C
     C* const line = lines + g * LS;
     const ArDP::W* tw = ArDP::table(p.tw, N);
     const bool convert = p.in_fmt == FMT_C128;
+    grid_wait();
 
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const TileGeom tg = tile_geom(p, tile, G);
+        if (tile + gridDim.x >= ntiles) grid_release();
         // the previous tile's store has read the staging area: copy this tile in
         const bool leader = CONTIG ? (w == 0 && lane == 0) : tid == 0;
         if (leader) bulk_wait_read_all();
@@ -382,8 +384,7 @@ cudaError_t launch_warp_tma_v(const StageLaunch& L, const CUtensorMap& map, cuda
     int64_t grid = (int64_t)L.sms * per_sm;
     if (grid > ntiles) grid = ntiles;
     if (grid < 1) grid = 1;
-    kern<<<(unsigned)grid, 32 * G * tma_wpl<N, G>(), smem, st>>>(L.args, ntiles, map);
-    return cudaGetLastError();
+    return launch_chained(kern, (unsigned)grid, 32 * G * tma_wpl<N, G>(), smem, st, L.args, ntiles, map);
 }
 
 // The asynchronous-output kernel for n = 256 / 512 and 4 or 8 lines per CTA,

@@ -130,6 +130,8 @@ __global__ void __launch_bounds__(kStageThreads) r2c_stage_kernel(const StageArg
     C* buf0 = reinterpret_cast<C*>(smem_raw);
     C* buf1 = buf0 + (size_t)n * ld;
     const int64_t L = p.M1, l0 = (int64_t)blockIdx.x * 2 * G;
+    grid_wait();
+    grid_release();
     const T* x = reinterpret_cast<const T*>(p.in);
     {   // real lines l0 + 2j, l0 + 2j + 1 -> complex line j
         const int dj = kStageThreads / n, di = kStageThreads - dj * n;
@@ -172,6 +174,8 @@ __global__ void __launch_bounds__(kStageThreads) c2r_stage_kernel(const StageArg
     C* buf0 = reinterpret_cast<C*>(smem_raw);
     C* buf1 = buf0 + (size_t)n * ld;
     const int64_t L = p.M1, l0 = (int64_t)blockIdx.x * 2 * G;
+    grid_wait();
+    grid_release();
     const typename RP::Scale ks = RP::scale_of(p.scale);
     {   // half lines l0 + 2j, l0 + 2j + 1 -> Hermitian-extended complex line j
         const int dj = kStageThreads / nh, dk = kStageThreads - dj * nh;
@@ -263,8 +267,10 @@ r2c_warp_kernel(const StageArgs p, int64_t ntiles)
     const int o = tid % TWO, slot = tid / TWO;          // store phase: line o of the tile
     const C* oline = tile + (o >> 1) * LS;
     int64_t t = blockIdx.x;
+    grid_wait();
     if (STAGED && t < ntiles) r2c_issue_raw<T, N>(x, L, t * TWO + 2 * warp, raw, lane);
     for (; t < ntiles; t += gridDim.x) {
+        if (t + gridDim.x >= ntiles) grid_release();
         const int64_t l0 = t * TWO;
         const int64_t la = l0 + 2 * warp, lb = la + 1;
         if constexpr (STAGED) {
@@ -355,8 +361,10 @@ c2r_warp_kernel(const StageArgs p, int64_t ntiles)
     const C* in = reinterpret_cast<const C*>(p.in);
     const typename RP::Scale ks = RP::scale_of(p.scale);
     int64_t t = blockIdx.x;
+    grid_wait();
     if (staged && t < ntiles) c2r_issue_raw<A, NH>(in, L, t * 2 * G + 2 * warp, raw, lane);
     for (; t < ntiles; t += gridDim.x) {
+        if (t + gridDim.x >= ntiles) grid_release();
         const int64_t la = t * 2 * G + 2 * warp, lb = la + 1;
         if (staged) {
             cp_async_wait_all();
@@ -419,9 +427,8 @@ cudaError_t launch_real_warp(const StageLaunch& L, cudaStream_t st)
     int64_t grid = (int64_t)L.sms * per_sm;
     if (grid > ntiles) grid = ntiles;
     if (grid < 1) grid = 1;
-    if (fwd) r2c_warp_kernel<A, N, G><<<(unsigned)grid, 32 * G, smem, st>>>(L.args, ntiles);
-    else c2r_warp_kernel<A, N, G><<<(unsigned)grid, 32 * G, smem, st>>>(L.args, ntiles);
-    return cudaGetLastError();
+    return fwd ? launch_chained(r2c_warp_kernel<A, N, G>, (unsigned)grid, 32 * G, smem, st, L.args, ntiles)
+               : launch_chained(c2r_warp_kernel<A, N, G>, (unsigned)grid, 32 * G, smem, st, L.args, ntiles);
 }
 
 template <class A>
@@ -445,7 +452,7 @@ cudaError_t launch_real_a(const StageLaunch& L, cudaStream_t st)
             if (e) return e;
             if (slot) *slot = 1;
         }
-        r2c_stage_kernel<A><<<grid, kStageThreads, L.smem, st>>>(L.args);
+        return launch_chained(r2c_stage_kernel<A>, grid, kStageThreads, L.smem, st, L.args);
     } else {
         int* slot = device_slot(attr_c2r);
         if (!slot || !*slot) {
@@ -454,9 +461,8 @@ cudaError_t launch_real_a(const StageLaunch& L, cudaStream_t st)
             if (e) return e;
             if (slot) *slot = 1;
         }
-        c2r_stage_kernel<A><<<grid, kStageThreads, L.smem, st>>>(L.args);
+        return launch_chained(c2r_stage_kernel<A>, grid, kStageThreads, L.smem, st, L.args);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace

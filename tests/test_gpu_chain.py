@@ -1,0 +1,75 @@
+"""Stages launched as a chain (a stage's CTAs may become resident while the stage
+before it drains): results of transforms enqueued back to back, on one stream, on two
+and replayed from a captured graph are bit for bit those of transforms run one at a
+time."""
+import numpy as np
+import pytest
+
+from paper_1501_07350_gb300 import openfft as of
+
+pytestmark = pytest.mark.gpu
+
+# kernels of every family: warp, asynchronous output (256, 512), any length, generic (2048)
+SHAPES = [(32, 32, 32), (64, 48, 100), (256, 32, 512), (36, 2048, 5)]
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch as _t
+    from paper_1501_07350_gb300 import _build
+    _build.build()
+    of.load()
+    assert _t.cuda.is_available()
+    return _t
+
+
+@pytest.mark.parametrize("dtype", [of.C2C_F64, of.C2C_F32])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_chained_transforms_match_single_ones(torch, shape, dtype):
+    tdt = torch.complex128 if dtype == of.C2C_F64 else torch.complex64
+    n = int(np.prod(shape))
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    plans = [of.Plan(*shape, 2, dtype, stream=s) for s in streams]
+    xs = [torch.randn(n, generator=gen, device="cuda", dtype=tdt) for _ in streams]
+    bufs = [[torch.empty_like(x) for _ in range(3)] for x in xs]
+    torch.cuda.synchronize()
+
+    def steps(i):
+        x, (y, z, w) = xs[i], bufs[i]
+        return [(x, y, of.FORWARD), (y, z, of.BACKWARD), (z, w, of.FORWARD)]
+
+    want = []
+    for i, p in enumerate(plans):
+        for a, b, d in steps(i):
+            p.exec(a, b, d)
+            torch.cuda.synchronize()
+        want.append([b.clone() for b in bufs[i]])
+
+    def check():
+        torch.cuda.synchronize()
+        for i in range(2):
+            for b, r in zip(bufs[i], want[i]):
+                assert torch.equal(torch.view_as_real(b), torch.view_as_real(r))
+                b.fill_(float("nan"))
+        torch.cuda.synchronize()
+
+    for _ in range(3):
+        for i, p in enumerate(plans):
+            for a, b, d in steps(i):
+                p.exec(a, b, d)
+    check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=streams[0]):
+        for a, b, d in steps(0):
+            plans[0].exec(a, b, d)
+    for i in range(2):
+        for b, r in zip(bufs[i], want[i]):
+            b.copy_(r)
+    bufs[0][2].fill_(float("nan"))
+    torch.cuda.synchronize()
+    graph.replay()
+    graph.replay()
+    check()
+    for p in plans:
+        p.close()
