@@ -62,8 +62,14 @@ struct ArF32 {
     __device__ __forceinline__ static C mul(C a, W w) {
         return make_float2(fmaf(a.x, w.x, -a.y * w.y), fmaf(a.x, w.y, a.y * w.x));
     }
-    // multiply by the complex constant re + i im
-    __device__ __forceinline__ static C mulc(C a, double re, double im) { return mul(a, make_float2((float)re, (float)im)); }
+    // multiply by the complex constant re + i im, its parts beyond binary32 included:
+    // with rounded constants every radix-16 butterfly turned its inputs by the same
+    // small error (256^3 1.78e-7 against 1.57e-7 relative, 1 % of the time)
+    __device__ __forceinline__ static C mulc(C a, double re, double im) {
+        const float rh = (float)re, ih = (float)im, rl = (float)(re - (double)rh), il = (float)(im - (double)ih);
+        return make_float2(fmaf(a.x, rh, fmaf(-a.y, ih, fmaf(a.x, rl, -a.y * il))),
+                           fmaf(a.x, ih, fmaf(a.y, rh, fmaf(a.x, il, a.y * rl))));
+    }
     __device__ __forceinline__ static C scale(C a, double k) {
         const float kf = (float)k;
         return make_float2(a.x * kf, a.y * kf);
