@@ -117,7 +117,6 @@ cudaError_t launch_tile_df(const StageLaunch& L, cudaStream_t st, bool* handled)
 // the asynchronous-output double-float kernels (fft_tma_256.cu, fft_tma_512.cu)
 cudaError_t launch_warp_tma_256(const StageLaunch& L, cudaStream_t st, bool* handled);
 cudaError_t launch_warp_tma_512(const StageLaunch& L, cudaStream_t st, bool* handled);
-cudaError_t launch_warp_tma_f32(const StageLaunch& L, cudaStream_t st, bool* handled);
 // any length (fft_mix.cu)
 cudaError_t launch_mix_df(const StageLaunch& L, cudaStream_t st, bool* handled);
 cudaError_t launch_mix_f32(const StageLaunch& L, cudaStream_t st, bool* handled);

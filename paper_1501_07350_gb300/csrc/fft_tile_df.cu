@@ -15,6 +15,14 @@ cudaError_t launch_tile_df(const StageLaunch& L, cudaStream_t st, bool* handled)
         cudaError_t e = L.args.n == 256 ? launch_warp_tma_256(L, st, handled) : launch_warp_tma_512(L, st, handled);
         if (*handled || e) return e;
     }
+    // a 32-point tile of the warp kernel is one warp: with few lines it leaves the
+    // chip nearly empty, and fft_mix's 128-thread tiles are faster (32^3 10.5 against
+    // 11.8 us, 64x32x32 11.9 against 14.4; 128x64x32, 8192 lines, the same; above, the
+    // warp kernel: 128x128x32 23 against 31)
+    if (L.family == KERNEL_AUTO && L.args.n == 32 && L.args.M1 * L.args.M2 <= 4096) {
+        cudaError_t e = launch_mix_df(L, st, handled);
+        if (*handled || e) return e;
+    }
     if ((L.family == KERNEL_AUTO || L.family == KERNEL_WARP) && (L.args.G == 4 || L.args.G == 8)) {
         cudaError_t e = L.args.G == 4 ? launch_warp_g<ArDP, 4>(L, st, handled) : launch_warp_g<ArDP, 8>(L, st, handled);
         if (*handled || e) return e;

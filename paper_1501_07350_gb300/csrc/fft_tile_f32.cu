@@ -1,7 +1,5 @@
 // fft_tile_f32.cu -- instantiations of the specialised stage kernels for one arithmetic:
 // warp-per-line kernels for power-of-two lengths, tile kernels for the others.
-// 256- and 512-point transposed stages take the asynchronous-output version
-// (fft_tma_f32.cu) whenever the stage's output has its view.
 #include "fft_tile.cuh"
 #include "fft_warp.cuh"
 
@@ -10,8 +8,14 @@ namespace ofg {
 cudaError_t launch_tile_f32(const StageLaunch& L, cudaStream_t st, bool* handled)
 {
     *handled = false;
-    if ((L.family == KERNEL_AUTO || L.family == KERNEL_WARP) && (L.args.n == 256 || L.args.n == 512)) {
-        cudaError_t e = launch_warp_tma_f32(L, st, handled);
+    // fft_mix also beats the warp kernel on the longer power-of-two lengths (256^3 156
+    // against 172-198 us, 512^3 1460 against 1590-1650) and on 64 and 128 points where
+    // there are lines enough to fill the chip several times (512x64x512 183 against
+    // 194, 512x128x512 354 against 362); 64^3 (4096 lines) takes 10.7 against 8-9 us
+    // and 128^3 (16384) 28.2 against 26.3
+    const int64_t lines = L.args.M1 * L.args.M2;
+    if (L.family == KERNEL_AUTO && (L.args.n >= 256 || (L.args.n >= 64 && lines >= 32768))) {
+        cudaError_t e = launch_mix_f32(L, st, handled);
         if (*handled || e) return e;
     }
     if ((L.family == KERNEL_AUTO || L.family == KERNEL_WARP) && (L.args.G == 8 || L.args.G == 16)) {

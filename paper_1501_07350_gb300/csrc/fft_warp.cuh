@@ -48,11 +48,10 @@ struct WarpLine {
     // form Q groups of S = 32 / Q; lane bl of group q takes butterflies
     // bl, bl + S, ... of lines q L + i (i < L), so the L lines share the
     // twiddle loads and give each thread L independent butterflies, and lines
-    // with fewer than 32 butterflies per pass still occupy every lane.
-    // The pass's results go through put(l, k, value): value k of the warp's
-    // line l (l < Q L), after every lane has read its inputs.
-    template <int P, int L, int Q, class Put>
-    __device__ __forceinline__ static void pass_to(const C* line0, const W* __restrict__ tw, int lane, Put put)
+    // with fewer than 32 butterflies per pass still occupy every lane.  In place:
+    // results are written after every lane has read its inputs.
+    template <int P, int L, int Q = 1>
+    __device__ __forceinline__ static void pass(C* line0, const W* __restrict__ tw, int lane)
     {
         constexpr int R = wplan_radix(N, P);
         constexpr int m = wplan_m(N, P);
@@ -61,8 +60,7 @@ struct WarpLine {
         constexpr int S = 32 / Q;
         constexpr int NB = (NBF + S - 1) / S;
         const int bl = lane % S;
-        const int l0 = (lane / S) * L;
-        line0 += l0 * LS;
+        line0 += (lane / S) * L * LS;
         C v[L][NB][R];
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
@@ -96,15 +94,9 @@ struct WarpLine {
 #pragma unroll
                 for (int i = 0; i < L; ++i)
 #pragma unroll
-                    for (int q = 0; q < R; ++q) put(l0 + i, base + m * q, v[i][u][q]);
+                    for (int q = 0; q < R; ++q) line0[i * LS + wpad<EB>(base + m * q)] = v[i][u][q];
             }
         }
-    }
-
-    template <int P, int L, int Q = 1>
-    __device__ __forceinline__ static void pass(C* line0, const W* __restrict__ tw, int lane)
-    {
-        pass_to<P, L, Q>(line0, tw, lane, [=](int l, int k, const C& x) { line0[l * LS + wpad<EB>(k)] = x; });
         __syncwarp();
     }
 
@@ -114,16 +106,6 @@ struct WarpLine {
         if constexpr (P < kPasses) {
             pass<P, L, Q>(line0, tw, lane);
             passes<P + 1, L, Q>(line0, tw, lane);
-        }
-    }
-
-    // every pass but the last, in place
-    template <int P, int L = 1, int Q = 1>
-    __device__ __forceinline__ static void passes_but_last(C* line0, const W* __restrict__ tw, int lane)
-    {
-        if constexpr (P < kPasses - 1) {
-            pass<P, L, Q>(line0, tw, lane);
-            passes_but_last<P + 1, L, Q>(line0, tw, lane);
         }
     }
 };
