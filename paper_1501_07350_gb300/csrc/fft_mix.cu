@@ -3,6 +3,7 @@
 #include "fft_mix.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <iterator>
 #include <vector>
 
@@ -92,28 +93,29 @@ MixLaunch make_launch(const int* radix, int count, float pass, int n)
     return l;
 }
 
-// of every length, made on the first launch
+// Each length's launch is made on its first use and kept (at most kMaxLen of them
+// per arithmetic and tile width); two threads may both make one, and one is kept.
 template <class A, int G>
 const MixLaunch& mix_launch(int n)
 {
-    static const std::vector<MixLaunch> all = [] {
-        constexpr bool df = sizeof(typename A::C) >= 16;
-        std::vector<MixLaunch> v(kMaxLen + 1);
-        v[0].plan.npass = v[1].plan.npass = 0;
-        for (int i = 2; i <= kMaxLen; ++i)
-            v[i] = df ? make_launch<A, G>(kRadixDF, (int)std::size(kRadixDF), i <= 64 ? 1.5f : (i <= 100 ? 3.5f : 6.5f), i)
-                      : make_launch<A, G>(kRadixF32, (int)std::size(kRadixF32), 100.f, i);
-        return v;
-    }();
-    return all[n];
+    static std::atomic<const MixLaunch*> made[kMaxLen + 1] = {};
+    const MixLaunch* l = made[n].load(std::memory_order_acquire);
+    if (l) return *l;
+    constexpr bool df = sizeof(typename A::C) >= 16;
+    const MixLaunch* mine =
+        new MixLaunch(df ? make_launch<A, G>(kRadixDF, (int)std::size(kRadixDF), n <= 64 ? 1.5f : (n <= 100 ? 3.5f : 6.5f), n)
+                         : make_launch<A, G>(kRadixF32, (int)std::size(kRadixF32), 100.f, n));
+    if (made[n].compare_exchange_strong(l, mine, std::memory_order_acq_rel)) return *mine;
+    delete mine;
+    return *l;
 }
 
-template <class A, int G>
-cudaError_t launch_mix_g(const StageLaunch& L, cudaStream_t st, bool* handled)
+template <class A, int G, bool REPEAT>
+cudaError_t launch_mix_r(const StageLaunch& L, cudaStream_t st, bool* handled)
 {
     const MixLaunch& ml = mix_launch<A, G>(L.args.n);
     if (ml.plan.npass == 0) return cudaSuccess;
-    auto kern = fft_mix_kernel<A, G>;
+    auto kern = fft_mix_kernel<A, G, REPEAT>;
     static int cached[kMaxDevices] = {};          // 1 once the kernel's attributes are set on the device
     int* slot = device_slot(cached);
     if (!slot || !*slot) {
@@ -122,13 +124,20 @@ cudaError_t launch_mix_g(const StageLaunch& L, cudaStream_t st, bool* handled)
         if (e) return e;
         if (slot) *slot = 1;
     }
-    *handled = true;
     StageArgs a = L.args;
     const int64_t Mg = a.group_i2 ? a.M2 : a.M1;
     a.ngroups = (Mg + G - 1) / G;
-    const int64_t ntiles = a.ngroups * (a.group_i2 ? a.M1 : a.M2);
+    const int64_t ntiles = a.ngroups * (a.group_i2 ? a.M1 : a.M2) * (REPEAT ? a.M3 : 1);
+    if (ntiles > 0x7fffffffLL) return cudaSuccess;      // tiles are counted in 32 bits
+    *handled = true;
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)L.sms * ml.per_sm, ntiles));
     return launch_chained(kern, (unsigned)grid, ml.threads, ml.smem, st, a, ml.plan, ntiles);
+}
+
+template <class A, int G>
+cudaError_t launch_mix_g(const StageLaunch& L, cudaStream_t st, bool* handled)
+{
+    return L.args.M3 > 1 ? launch_mix_r<A, G, true>(L, st, handled) : launch_mix_r<A, G, false>(L, st, handled);
 }
 
 }  // namespace

@@ -190,7 +190,7 @@ struct Mix {
     }
 };
 
-template <class A, int G>
+template <class A, int G, bool REPEAT>
 __global__ void __launch_bounds__(kMixMaxThreads, mix_min_ctas())
 fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t ntiles)
 {
@@ -204,13 +204,13 @@ fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t 
     const int tid = threadIdx.x, T = blockDim.x;
     const int g = M::line_of(tid), slot = M::slot_of(tid), slots = plan.slots, at = g * ld;
     int64_t tile = blockIdx.x;
-    TileGeom tg = tile_geom(p, tile, G);                // the grid has at most ntiles CTAs
+    TileGeom tg = tile_geom<REPEAT>(p, tile, G);                // the grid has at most ntiles CTAs
     grid_wait();
     for (int i = tid; i < p.n; i += T) cp_async<M::E>(tw + i, reinterpret_cast<const C*>(p.tw) + i);
     M::issue_load(p, tg.line0, tg.lstride, tg.valid, cur, ld, tid, T);
     for (; tile < ntiles; tile += gridDim.x) {
         const int64_t next = tile + gridDim.x;
-        const TileGeom tn = tile_geom(p, next < ntiles ? next : tile, G);
+        const TileGeom tn = tile_geom<REPEAT>(p, next < ntiles ? next : tile, G);
         if (next >= ntiles) grid_release();
         const bool mine = g < tg.valid;
         cp_async_wait_all();

@@ -156,7 +156,7 @@ int* fallback_status_word()
 cudaError_t launch_stage(const StageLaunch& L0, cudaStream_t st)
 {
     StageLaunch L = L0;
-    const int64_t elems = L.args.M1 * L.args.M2 * (int64_t)L.args.n;
+    const int64_t elems = L.args.M1 * L.args.M2 * (L.args.M3 > 1 ? L.args.M3 : 1) * (int64_t)L.args.n;
     if (!L.args.in_elems) L.args.in_elems = elems;
     if (!L.args.out_elems) L.args.out_elems = elems;
     if (!L.args.chk) L.args.chk = L.status ? L.status : fallback_status_word();
@@ -164,6 +164,28 @@ cudaError_t launch_stage(const StageLaunch& L0, cudaStream_t st)
     if (L.arith == ARITH_TC_TF32 || L.arith == ARITH_TC_BF16) return launch_dftgemm(L, st, L.status);
     bool handled = false;
     cudaError_t e = cudaSuccess;
+    if (L.args.M3 > 1) {
+        // a geometry repeated over i3: one launch of the any-length kernel, or one
+        // launch per i3 where each fills the chip and the length has a faster kernel
+        // (double-float powers of two)
+        const bool own = L.arith == ARITH_DF && warp_length(L.args.n) && L.args.M1 * L.args.M2 >= 16384;
+        if (!own && L.family == KERNEL_AUTO) {
+            e = L.arith == ARITH_F32 ? launch_mix_f32(L, st, &handled) : launch_mix_df(L, st, &handled);
+            if (handled || e) return e;
+        }
+        StageLaunch one = L;
+        const int64_t lines = L.args.M1 * L.args.M2 * (int64_t)L.args.n, E = L.arith == ARITH_F32 ? 8 : 16;
+        one.args.M3 = 1;
+        one.grid = L.args.ngroups * (L.args.group_i2 ? L.args.M1 : L.args.M2);
+        for (int64_t i3 = 0; i3 < L.args.M3 && !e; ++i3) {
+            one.args.in = static_cast<const char*>(L.args.in) + i3 * lines * E;
+            one.args.out = static_cast<char*>(L.args.out) + i3 * L.args.S3 * E;
+            one.args.in_elems = L.args.in_elems - i3 * lines;
+            one.args.out_elems = L.args.out_elems - i3 * L.args.S3;
+            e = launch_stage(one, st);
+        }
+        return e;
+    }
     if (L.args.do_fft && L.family != KERNEL_GENERIC) {
         switch (L.arith) {
         case ARITH_F64: e = launch_tile_f64(L, st, &handled); break;

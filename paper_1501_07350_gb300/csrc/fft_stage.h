@@ -21,13 +21,15 @@ enum { ARITH_F64 = 0, ARITH_F32 = 1, ARITH_DF = 2, ARITH_TC_TF32 = 3, ARITH_TC_B
 // of length n at in + l * n.  Output element (l, k) goes to
 // out[i1 * S1 + i2 * S2 + k * Sk].  A CTA takes G consecutive values of i1
 // (group_i2 = 0) or of i2 (group_i2 = 1), the coordinate whose output stride
-// is 1, so a store at fixed k writes G consecutive elements.
+// is 1, so a store at fixed k writes G consecutive elements.  With M3 > 1 that
+// geometry repeats: line l + i3 M1 M2, out + i3 S3, for i3 < M3 (0 stands for 1).
 struct StageArgs {
     const void* in;
     void* out;
     const void* tw;            // twiddle table of length n (W[e] = exp(-2 pi i e / n))
     const void* aux;           // DFT-GEMM stages: operand image of the DFT matrices
     int64_t M1, M2, S1, S2, Sk;
+    int64_t M3, S3;
     int64_t ngroups;           // ceil(M_grouped / G)
     double scale;              // applied at store (1.0 = none)
     int n, G, log2G;

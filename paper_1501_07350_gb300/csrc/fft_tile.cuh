@@ -119,6 +119,10 @@ struct TileGeom {
     int valid;
 };
 
+// REPEAT: the geometry repeats over i3 (StageArgs M3 > 1).  Kernels that do not take
+// it are launched once per i3 (launch_stage): the extra division and registers
+// cost the asynchronous-output kernel 1.4 % of every transform.
+template <bool REPEAT = false>
 __device__ __forceinline__ TileGeom tile_geom(const StageArgs& p, int64_t tile, int G)
 {
     TileGeom t;
@@ -134,6 +138,12 @@ __device__ __forceinline__ TileGeom tile_geom(const StageArgs& p, int64_t tile, 
         grp = tile - outer * p.ngroups;
     }
     const int64_t first = grp * G;
+    int64_t i3 = 0;
+    if constexpr (REPEAT) {
+        const uint32_t Mo = (uint32_t)(p.group_i2 ? p.M1 : p.M2);
+        i3 = (uint32_t)outer / Mo;                 // launch grids fit 31 bits
+        outer -= i3 * Mo;
+    }
     if (!p.group_i2) {
         t.line0 = first + outer * p.M1; t.lstride = 1;
         t.obase = first * p.S1 + outer * p.S2; t.ostride = p.S1;
@@ -142,6 +152,10 @@ __device__ __forceinline__ TileGeom tile_geom(const StageArgs& p, int64_t tile, 
         t.line0 = outer + first * p.M1; t.lstride = p.M1;
         t.obase = outer * p.S1 + first * p.S2; t.ostride = p.S2;
         t.valid = (int)(p.M2 - first < G ? p.M2 - first : G);
+    }
+    if constexpr (REPEAT) {
+        t.line0 += i3 * p.M1 * p.M2;
+        t.obase += i3 * p.S3;
     }
     return t;
 }

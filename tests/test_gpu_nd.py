@@ -98,3 +98,28 @@ def test_nd_errors(torch):
         assert ei.value.status == of.ERR_ALIAS
     finally:
         of.openfft_nd_destroy(plan)
+
+
+# The middle stages of the backward transform repeat a two-coordinate line geometry
+# over the slower axes (one launch): each stage kernel on such an axis, ragged tiles
+# (5, 6 or 9 grouped lines), one and two slower axes.
+@pytest.mark.parametrize("dtype", [of.C2C_F64, of.C2C_F32])
+@pytest.mark.parametrize("dims", [(3, 256, 9, 4), (2, 512, 5, 3), (3, 64, 6, 7), (5, 36, 9, 6), (4, 225, 2, 3),
+                                  (2, 3, 256, 9, 2), (3, 2, 32, 5, 4), (2, 2048, 3, 2), (2, 5, 30, 6, 7)])
+def test_repeated_line_geometry(torch, dims, dtype):
+    x = synth.complex_field(dims, seed=int(np.prod(dims)))
+    tol = 1e-12 if dtype == of.C2C_F64 else 1e-5
+    tdt = torch.complex128 if dtype == of.C2C_F64 else torch.complex64
+    xin = x if dtype == of.C2C_F64 else x.astype(np.complex64).astype(np.complex128)
+    plan = of.openfft_nd_plan(dims, 1, dtype)
+    try:
+        of.openfft_nd_set_stream(plan, torch.cuda.current_stream())
+        xd = torch.from_numpy(np.ascontiguousarray(xin.reshape(-1))).to(device="cuda", dtype=tdt)
+        for direction, odir in ((of.FORWARD, oracle.FORWARD), (of.BACKWARD, oracle.BACKWARD)):
+            yd = torch.full_like(xd, float("nan"))
+            of.openfft_nd_exec(plan, xd, yd, direction)
+            torch.cuda.synchronize()
+            ref = oracle.fftnd(xin, dims, 1, odir)
+            assert oracle.rel_l2(yd.cpu().numpy().astype(np.complex128), ref) < tol, (dims, direction)
+    finally:
+        of.openfft_nd_destroy(plan)
