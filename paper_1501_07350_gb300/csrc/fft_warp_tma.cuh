@@ -1,5 +1,5 @@
 // fft_warp_tma.cuh -- the double-float warp-per-line stage kernel with an
-// asynchronous output path, for 256- and 512-point lines in tiles of 4 or 8.
+// asynchronous output path, for 256- and 512-point lines in tiles of 4.
 //
 // The radix passes are those of fft_warp.cuh (packed double-float policy,
 // per-pass twiddle tables).  What differs is the output: the last radix pass
@@ -10,9 +10,8 @@
 // Transposed output (the fused transposes of steps (4)-(6), Sec. 3.1.1): the
 // tile's G lines are consecutive in the output at every frequency k, so the
 // staging area is [k][G lines] of 16-byte elements in the swizzle of the
-// tensor store (rows of 128 bytes, 16-byte chunk index XOR row mod 8, for
-// G = 8; rows of 64 bytes, chunk XOR (row / 2) mod 4, for G = 4), which also
-// keeps the last pass's shared-memory writes free of bank conflicts.  The
+// tensor store (rows of 64 bytes, 16-byte chunk index XOR (row / 2) mod 4), which
+// also keeps the last pass's shared-memory writes free of bank conflicts.  The
 // tensor map views the output as (grouped line coordinate, frequency, other
 // line coordinate) with element strides (1, Sk, So).
 //
@@ -64,23 +63,22 @@ __device__ __forceinline__ void line_sync(int g)
 // warps per line.  512-point lines take two: each lane then holds one
 // radix-8 butterfly (8 values) instead of two, which halves the registers a
 // thread needs (64) and doubles the resident warps per SM (32) for the same
-// shared memory; measured 5 % faster on 512^3 than one warp per line (4-line
-// CTAs), 4 % with 8-line CTAs.  256-point lines keep one: their 4 x 8 x 8 plan
+// shared memory; measured 5 % faster on 512^3 than one warp per line.  256-point lines keep one: their 4 x 8 x 8 plan
 // has 32 radix-8 butterflies per pass, and a second warp would idle there.
-template <int N, int G>
+template <int N>
 constexpr int tma_wpl() { return N == 512 ? 2 : 1; }
 // CTAs per SM the register allocation is sized for: 64 registers a thread,
 // 32 warps per SM
-template <int N, int G>
-constexpr int tma_min_ctas() { return G == 8 ? (N == 512 ? 2 : 4) : (N == 256 ? 8 : 4); }
+template <int N>
+constexpr int tma_min_ctas() { return N == 256 ? 8 : 4; }
 
 // byte offset of output element (frequency k, tile line g) in the transposed
 // staging area: the tensor store's swizzle for rows of G x 16 bytes
 template <int G>
 __device__ __forceinline__ uint32_t staged_offset(int k, int g)
 {
-    if constexpr (G == 8) return (uint32_t)k * 128u + ((uint32_t)(g ^ (k & 7)) << 4);
-    else return (uint32_t)k * 64u + ((uint32_t)(g ^ ((k >> 1) & 3)) << 4);
+    static_assert(G == 4, "rows of 64 bytes");
+    return (uint32_t)k * 64u + ((uint32_t)(g ^ ((k >> 1) & 3)) << 4);
 }
 
 template <int N, int WPL>
@@ -247,10 +245,10 @@ template <int N, int G>
 constexpr size_t tma_smem_bytes() { return 1024 + (size_t)G * warp_line_stride<16>(N) * 16; }
 
 template <int N, int G, bool CONTIG, bool CONJ_SCALE, bool EXT>
-__global__ void __launch_bounds__(32 * G * tma_wpl<N, G>(), tma_min_ctas<N, G>())
+__global__ void __launch_bounds__(32 * G * tma_wpl<N>(), tma_min_ctas<N>())
 fft_warp_tma_kernel(const StageArgs p, int64_t ntiles, const __grid_constant__ CUtensorMap tmap)
 {
-    constexpr int WPL = tma_wpl<N, G>();
+    constexpr int WPL = tma_wpl<N>();
     using L = TmaLine<N, WPL>;
     using C = ArDP::C;
     constexpr int LS = L::LS;
@@ -300,19 +298,10 @@ fft_warp_tma_kernel(const StageArgs p, int64_t ntiles, const __grid_constant__ C
         }
         __syncthreads();
         if (tid == 0) {
-            if constexpr (!CONTIG) {
 #pragma unroll
-                for (int kb = 0; kb < (N + 255) / 256; ++kb)
-                    tma_store_3d(&tmap, smem_addr(stage) + (uint32_t)kb * 256u * (uint32_t)(G * 16),
-                                 (int)((tile % p.ngroups) * G * 4), kb * 256, (int)(tile / p.ngroups));
-            } else {
-                char* first = reinterpret_cast<char*>(p.out) + tg.obase * 16;
-                for (int gg = 0; gg < tg.valid; ++gg)
-                    if (in_bounds(p.chk, tg.obase + gg * tg.ostride, p.out_elems) &&
-                        in_bounds(p.chk, tg.obase + gg * tg.ostride + N - 1, p.out_elems))
-                        bulk_store(first + (int64_t)gg * tg.ostride * 16, smem_addr(stage) + (uint32_t)gg * N * 16u,
-                                   N * 16u);
-            }
+            for (int kb = 0; kb < (N + 255) / 256; ++kb)
+                tma_store_3d(&tmap, smem_addr(stage) + (uint32_t)kb * 256u * (uint32_t)(G * 16),
+                             (int)((tile % p.ngroups) * G * 4), kb * 256, (int)(tile / p.ngroups));
             bulk_commit();
         }
     }
@@ -344,7 +333,7 @@ inline TensorMapEncodeFn tensor_map_encoder()
 }
 
 // The transposed output as a 3-D tensor of 4-byte words: (grouped line
-// coordinate x 4, frequency, other line coordinate); box (8 lines, 256 or n
+// coordinate x 4, frequency, other line coordinate); box (G lines, 256 or n
 // frequencies, 1).  false if the stage's geometry has no such view.
 inline bool transposed_store_map(const StageArgs& a, int G, CUtensorMap* map)
 {
@@ -362,7 +351,7 @@ inline bool transposed_store_map(const StageArgs& a, int G, CUtensorMap* map)
     const cuuint32_t box[3] = {(cuuint32_t)(4 * G), (cuuint32_t)(a.n < 256 ? a.n : 256), 1u};
     const cuuint32_t estr[3] = {1u, 1u, 1u};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, a.out, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               G == 8 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
            CUDA_SUCCESS;
 }
@@ -376,7 +365,7 @@ cudaError_t launch_warp_tma_v(const StageLaunch& L, const CUtensorMap& map, cuda
     int* slot = device_slot(cached);
     int per_sm = slot ? *slot : 0;
     if (per_sm == 0) {
-        cudaError_t e = persistent_ctas_per_sm((const void*)kern, 32 * G * tma_wpl<N, G>(), smem, &per_sm);
+        cudaError_t e = persistent_ctas_per_sm((const void*)kern, 32 * G * tma_wpl<N>(), smem, &per_sm);
         if (e) return e;
         if (slot) *slot = per_sm;
     }
@@ -384,15 +373,19 @@ cudaError_t launch_warp_tma_v(const StageLaunch& L, const CUtensorMap& map, cuda
     int64_t grid = (int64_t)L.sms * per_sm;
     if (grid > ntiles) grid = ntiles;
     if (grid < 1) grid = 1;
-    return launch_chained(kern, (unsigned)grid, 32 * G * tma_wpl<N, G>(), smem, st, L.args, ntiles, map);
+    return launch_chained(kern, (unsigned)grid, 32 * G * tma_wpl<N>(), smem, st, L.args, ntiles, map);
 }
 
-// The asynchronous-output kernel for n = 256 / 512 and 4 or 8 lines per CTA,
+// The asynchronous-output kernel for n = 256 / 512 in tiles of G lines,
 // when the stage's output has the view it needs; *handled = false otherwise.
 template <int N, int G>
-cudaError_t launch_warp_tma_n(const StageLaunch& L, cudaStream_t st, bool* handled)
+cudaError_t launch_warp_tma_n(const StageLaunch& L0, cudaStream_t st, bool* handled)
 {
-    const StageArgs& a = L.args;
+    StageLaunch L = L0;
+    StageArgs& a = L.args;
+    a.G = G;
+    a.ngroups = ((a.group_i2 ? a.M2 : a.M1) + G - 1) / G;
+    L.grid = a.ngroups * (a.group_i2 ? a.M1 : a.M2);
     CUtensorMap map;
     std::memset(&map, 0, sizeof(map));
     const bool contig = a.contig_store != 0;
