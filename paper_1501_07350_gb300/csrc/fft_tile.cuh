@@ -126,17 +126,11 @@ template <bool REPEAT = false>
 __device__ __forceinline__ TileGeom tile_geom(const StageArgs& p, int64_t tile, int G)
 {
     TileGeom t;
-    // 32-bit division whenever the operands fit (launch grids always do):
-    // the 64-bit one is a long software sequence run twice per tile
-    int64_t outer, grp;
-    if (((uint64_t)tile | (uint64_t)p.ngroups) >> 32 == 0) {
-        const uint32_t o = (uint32_t)tile / (uint32_t)p.ngroups;
-        outer = o;
-        grp = (int64_t)((uint32_t)tile - o * (uint32_t)p.ngroups);
-    } else {
-        outer = tile / p.ngroups;
-        grp = tile - outer * p.ngroups;
-    }
+    // tiles are counted in 31 bits (the launch grids are checked): 32-bit division;
+    // with a 64-bit path beside it 256^3 complex128 took 1.2 % longer
+    const uint32_t o = (uint32_t)tile / (uint32_t)p.ngroups;
+    int64_t outer = o;
+    const int64_t grp = (int64_t)((uint32_t)tile - o * (uint32_t)p.ngroups);
     const int64_t first = grp * G;
     int64_t i3 = 0;
     if constexpr (REPEAT) {
