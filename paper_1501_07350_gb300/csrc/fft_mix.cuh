@@ -78,16 +78,18 @@ struct Mix {
     __device__ __forceinline__ static int slot_of(int tid) { return kPairs ? (tid & 1) + 2 * (tid / (2 * G)) : tid / G; }
 
     // Copies of a tile: `valid` lines, lstride apart from line0 on, a warp per line
-    // in 16-byte pieces (8 bytes where an odd length leaves lines unaligned).
+    // in 16-byte pieces (8 bytes where an odd length or the array's address leaves
+    // lines of complex64 unaligned).
     __device__ __forceinline__ static void issue_load(const StageArgs& p, int64_t line0, int64_t lstride, int valid, C* buf,
                                                       int ld, int tid, int T)
     {
         const int n = p.n, lane = tid & 31;
+        const bool wide = ((n & 1) | (int)(reinterpret_cast<uintptr_t>(p.in) & 15)) == 0;
         for (int g = tid >> 5; g < valid; g += T >> 5) {
             const int64_t e = (line0 + g * lstride) * n;
             const char* src = reinterpret_cast<const char*>(p.in) + e * E;
             C* dst = buf + g * ld;
-            if (E == 16 || (n & 1)) {
+            if (E == 16 || !wide) {
 #pragma unroll 4
                 for (int i = lane; i < n; i += 32)
                     if (in_bounds(p.chk, e + i, p.in_elems)) cp_async<E>(dst + i, src + i * E);

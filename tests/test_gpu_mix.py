@@ -57,3 +57,25 @@ def test_every_radix_and_position(torch, n, dtype):
                 assert err < TOL[dtype], (shape, direction, err)
         finally:
             of.openfft_destroy(plan)
+
+
+@pytest.mark.parametrize("shape", [(36, 10, 48), (9, 25, 14), (256, 6, 80)])
+def test_complex64_arrays_at_8_byte_addresses(torch, shape):
+    """complex64 arrays that start 8 bytes off a 16-byte boundary (a view into a larger
+    tensor): the copies of a line then take 8 bytes at a time."""
+    n = int(np.prod(shape))
+    x = synth.complex_field(shape, seed=n).astype(np.complex64)
+    plan = of.openfft_plan(*shape, 1, of.C2C_F32)
+    try:
+        of.openfft_set_stream(plan, torch.cuda.current_stream())
+        for off_in, off_out in ((1, 0), (0, 1), (1, 1)):
+            xd = torch.empty(n + 1, dtype=torch.complex64, device="cuda")[off_in:off_in + n]
+            xd.copy_(torch.from_numpy(x.reshape(-1)))
+            yd = torch.full((n + 1,), float("nan"), dtype=torch.complex64, device="cuda")[off_out:off_out + n]
+            for direction, odir in ((of.FORWARD, oracle.FORWARD), (of.BACKWARD, oracle.BACKWARD)):
+                ref = oracle.fft3d(x.astype(np.complex128), *shape, 1, odir)
+                of.openfft_exec_c2c(plan, xd, yd, direction)
+                of.openfft_sync(plan)
+                assert oracle.rel_l2(yd.cpu().numpy().astype(np.complex128), ref) < TOL[of.C2C_F32]
+    finally:
+        of.openfft_destroy(plan)
