@@ -165,6 +165,10 @@ constexpr double kS73 = 0.43388373911755812047576833284835875461;     // sin(6 p
 
 template <class A, int R> struct Dft;
 
+template <class A> struct Dft<A, 1> {
+    __device__ __forceinline__ static void run(typename A::C*) {}
+};
+
 template <class A> struct Dft<A, 2> {
     __device__ __forceinline__ static void run(typename A::C* x) {
         auto t = A::sub(x[0], x[1]);

@@ -1,9 +1,8 @@
 // batch.cu -- many 3-D transforms of uneven sizes in one persistent launch,
 // replayed from a captured CUDA graph.
 //
-// Work items are runs of up to kTilesPerItem (16) tiles (of G lines each) of one
-// stage of one transform, handed out
-// in stage-major order (every stage-1 tile of every transform, then every
+// Work items are runs of tiles (of G lines each) of one stage of
+// one transform, handed out in stage-major order (every stage-1 tile of every transform, then every
 // stage-2 tile, then every stage-3 tile) through one atomic queue head.  A
 // stage-s item of transform i first waits until all stage-(s-1) tiles of
 // transform i are done (a per-(stage, transform) counter).  Those items have
@@ -13,11 +12,20 @@
 // OPENFFT_ERR_TIMEOUT in a status word, every CTA stops taking items, and the
 // host reads the status at openfft_sync.
 //
-// Per item the CTA runs the same stage computation as the single-transform
-// path: compile-time-specialised tile bodies for the common lengths, the
-// generic body otherwise.  Data written by one CTA and read by another in a
-// later stage is loaded with cp.async.cg (through L2, not L1) after an
-// acquire on the counter; writers fence before releasing.
+// Per item the CTA runs the any-length stage computation (fft_mix.cuh) with the
+// length's radix plan.  Data written by one CTA and read by another in a later stage
+// is loaded with cp.async (after an acquire on the counter, and by a launch whose L1
+// holds no older copy of it); writers fence before releasing.
+//
+// The time is the tiles': small CTAs (128 threads, up to 8 per SM) keep copies, passes
+// and stores of different items in flight.  64 uneven complex64 transforms (48^3 to
+// 100x108x120) take 461 us, 797 with 256-thread CTAs and the specialised tile bodies
+// (272 would be three reads and writes at the measured copy rate); the same in
+// double-float 1534, 3253 before.  A CTA claims its next
+// item before it starts on the current one, so the queue's atomic and the search are
+// not waited for.  A claimed item may stay behind one that waits for earlier items;
+// waits still end: the unfinished item with the lowest index is never behind another,
+// and everything it waits for has lower indices.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -26,202 +34,30 @@
 #include "../../include/openfft_gb.h"
 #include "batch.h"
 #include "fft_stage.h"
-#include "fft_tile.cuh"
-#include "generic_stage.cuh"
+#include "batch_kernel.cuh"
 
 namespace ofg {
 
-constexpr int kBatchThreads = 256;
-constexpr int kTilesPerItem = 16;          // tiles of one (stage, transform) per work item (the
-                                           // queue and dependency work of an item is serial)
-
-struct BatchCounters {
-    unsigned long long next;   // queue head
-    int status;                // OPENFFT_OK or OPENFFT_ERR_TIMEOUT
-    int pad;
-    // followed by done[3 * count]
-};
-
-struct BatchDev {
-    const StageArgs* stages;       // [2 directions][3 stages][count]
-    const int64_t* item_base;      // [3 * count + 1]: queue index of the first tile of (stage, transform)
-    const unsigned* need;          // [3 * count]: tiles of (stage, transform)
-    void* const* ptrs;             // [2 * count]: in_i, out_i (device pointers)
-    void* const* scratch;          // [count]
-    BatchCounters* ctr;
-    unsigned* done;                // [3 * count]
-    int count;
-    int dir_index;                 // 0 forward, 1 backward
-    long long wait_budget;         // clock64 cycles
-};
-
-// Tiles [t0, t1) of one stage of one transform; the next tile's lines are
-// copied into the second buffer while the current tile is transformed.
-template <class A, int N, int G>
-__device__ __noinline__ void tile_item(const StageArgs& p, int64_t t0, int64_t t1, typename A::C* buf,
-                                       int tid)
-{
-    using C = typename A::C;
-    constexpr int T = kBatchThreads;
-    C* cur = buf;
-    C* nxt = buf + Tile<A, N, G, T>::kElems;
-    const bool convert = Io<A>::kConverts && p.in_fmt == FMT_C128;
-    tile_issue_loads<A, N, G, T>(p, tile_geom(p, t0, G), cur, tid);
-    for (int64_t t = t0; t < t1; ++t) {
-        const TileGeom tg = tile_geom(p, t, G);
-        cp_async_wait_all();
-        if (convert) { if (p.conj_in) tile_fix<A, N, G, T, true, true>(cur, tid); else tile_fix<A, N, G, T, true, false>(cur, tid); }
-        else if (p.conj_in) tile_fix<A, N, G, T, false, true>(cur, tid);
-        __syncthreads();
-        if (t + 1 < t1) tile_issue_loads<A, N, G, T>(p, tile_geom(p, t + 1, G), nxt, tid);
-        Tile<A, N, G, T>::template passes<0>(cur + tid % G, reinterpret_cast<const typename A::W*>(p.tw), tid / G);
-        tile_store_dispatch<A, N, G, T>(p, tg, cur, tid);
-        __syncthreads();
-        C* x = cur; cur = nxt; nxt = x;
-    }
-    cp_async_wait_all();
-}
-
-// the tile bodies are compiled for G lines per tile; contiguous tile stores
-// assume the lines of the output in order
-template <int G>
-__device__ __forceinline__ bool tile_ok(const StageArgs& p)
-{
-    return p.G == G && (!p.contig_store || (!p.group_i2 && p.S1 == p.n && p.Sk == 1));
-}
-
-// Shared-memory layout of the batched kernel: [tile buffer | queue prefix
-// item_base (3 count + 1 int64) | tile counts need (3 count uint32)].
-template <class A, int G>
-__global__ void __launch_bounds__(kBatchThreads, sizeof(typename A::C) == 8 ? 3 : 2)
-batch_kernel(const BatchDev d, size_t buf_bytes)
-{
-    using C = typename A::C;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int64_t s_in[kMaxLinesPerCta];
-    __shared__ int64_t s_out[kMaxLinesPerCta];
-    __shared__ StageArgs s_p;
-    __shared__ int64_t s_tile;        // first tile of the item
-    __shared__ int s_q, s_abort;
-    const int tid = threadIdx.x;
-    const int nq = 3 * d.count;
-    int64_t* sh_base = reinterpret_cast<int64_t*>(smem_raw + buf_bytes);
-    unsigned* sh_need = reinterpret_cast<unsigned*>(sh_base + nq + 1);
-    for (int k = tid; k <= nq; k += kBatchThreads) sh_base[k] = d.item_base[k];
-    for (int k = tid; k < nq; k += kBatchThreads) sh_need[k] = d.need[k];
-    __syncthreads();
-    const int64_t total = sh_base[nq];
-    volatile int* status = &d.ctr->status;
-
-    for (;;) {
-        if (tid == 0) {
-            const int64_t j = (int64_t)atomicAdd(&d.ctr->next, 1ull);
-            int abort = *status != OPENFFT_OK || j >= total;
-            int q = 0;
-            if (!abort) {
-                // (stage, transform) of item j: last q with item_base[q] <= j
-                int lo = 0, hi = nq - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (sh_base[mid] <= j) lo = mid; else hi = mid - 1;
-                }
-                q = lo;
-                const int s = q / d.count;
-                if (s > 0) {
-                    volatile unsigned* cnt = &d.done[q - d.count];
-                    const unsigned want = sh_need[q - d.count];
-                    const long long t0 = clock64();
-                    while (*cnt < want) {
-                        if (*status != OPENFFT_OK) { abort = 1; break; }
-                        if (clock64() - t0 > d.wait_budget) {
-                            atomicCAS(&d.ctr->status, OPENFFT_OK, OPENFFT_ERR_TIMEOUT);
-                            abort = 1;
-                            break;
-                        }
-                        __nanosleep(128);
-                    }
-                    __threadfence();               // acquire: order the loads after the counter
-                }
-            }
-            s_abort = abort;
-            s_q = q;
-            s_tile = abort ? 0 : (j - sh_base[q]) * kTilesPerItem;
-        }
-        __syncthreads();
-        if (s_abort) break;
-        const int q = s_q, s = q / d.count, i = q - s * d.count;
-        // stage descriptor of (stage, transform) into shared memory, pointers patched
-        if (tid < (int)(sizeof(StageArgs) / 4)) {
-            reinterpret_cast<int*>(&s_p)[tid] = __ldg(reinterpret_cast<const int*>(&d.stages[d.dir_index * nq + q]) + tid);
-        }
-        __syncthreads();
-        if (tid == 0) {
-            void* in_i = d.ptrs[2 * i];
-            void* out_i = d.ptrs[2 * i + 1];
-            void* sc = d.scratch[i];
-            s_p.in = s == 0 ? in_i : (s == 1 ? sc : out_i);
-            s_p.out = s == 0 ? sc : out_i;
-        }
-        __syncthreads();
-        const StageArgs& p = s_p;
-        const int64_t t0 = s_tile;
-        const int64_t ntile = p.ngroups * (p.group_i2 ? p.M1 : p.M2);
-        const int64_t t1 = t0 + kTilesPerItem < ntile ? t0 + kTilesPerItem : ntile;
-        C* buf = reinterpret_cast<C*>(smem_raw);
-        bool done_item = false;
-        if (tile_ok<G>(p)) {
-            done_item = true;
-            switch (p.n) {
-            case 48: tile_item<A, 48, G>(p, t0, t1, buf, tid); break;
-            case 64: tile_item<A, 64, G>(p, t0, t1, buf, tid); break;
-            case 96: tile_item<A, 96, G>(p, t0, t1, buf, tid); break;
-            case 100: tile_item<A, 100, G>(p, t0, t1, buf, tid); break;
-            case 108: tile_item<A, 108, G>(p, t0, t1, buf, tid); break;
-            case 120: tile_item<A, 120, G>(p, t0, t1, buf, tid); break;
-            default: done_item = false; break;
-            }
-        }
-        if (!done_item)
-            for (int64_t t = t0; t < t1; ++t) {
-                generic_stage_tile<A>(p, t, smem_raw, s_in, s_out);
-                __syncthreads();
-            }
-        __threadfence();                           // release this thread's stores
-        __syncthreads();
-        if (tid == 0) atomicAdd(&d.done[q], 1u);
-    }
-}
+// Tiles of one (stage, transform) per work item: enough that an item's queue and
+// descriptor work is small beside them, few enough that a stage of the batch is about
+// kItemsPerCta items for every CTA: eight 128^3 complex64 transforms take 182 us (245
+// with 16 tiles an item), 64 uneven ones 461 (472 with four items per CTA, 495 six).
+constexpr int kMaxTilesPerItem = 16;
+constexpr int kItemsPerCta = 2;
 
 // --------------------------------------------------------------- host ----
 
-namespace {
-
-bool radix_plan(int n, StageArgs& a)
-{
-    int m = n, c = 0;
-    const int rs[6] = {8, 4, 2, 3, 5, 7};
-    for (int r : rs)
-        while (m % r == 0) {
-            if (c >= kMaxPasses) return false;
-            a.radix[c++] = r;
-            m /= r;
-        }
-    a.npass = c;
-    return m == 1;
-}
-
-int lg2(int g) { int l = 0; while ((1 << l) < g) ++l; return l; }
-
-}  // namespace
+size_t tile_bytes_of(bool f32, int G, int n) { return f32 ? batch_tile_bytes_f32(G, n) : batch_tile_bytes_df(G, n); }
+const void* kernel_of(bool f32, int G) { return f32 ? batch_kernel_f32(G) : batch_kernel_df(G); }
 
 struct BatchPlan {
-    int count = 0, dtype = 0, arith = 0, G = 8;
+    int count = 0, dtype = 0, arith = 0, G = 8, tiles_per_item = 1;
     std::vector<int> dims;                     // 3 * count
     std::vector<int64_t> N;                    // per transform
     size_t smem = 0;
     int grid = 0;
     // device memory
-    StageArgs* d_stages = nullptr;
+    StageArgs* d_stages = nullptr;             // and the radix plans after them
     int64_t* d_item_base = nullptr;
     unsigned* d_need = nullptr;
     void** d_ptrs = nullptr;
@@ -268,7 +104,6 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
     b->count = count;
     b->dtype = dtype;
     b->arith = dtype == OPENFFT_C2C_F32 ? ARITH_F32 : ARITH_DF;
-    b->G = dtype == OPENFFT_C2C_F32 ? 16 : 8;
     b->dims.assign(dims, dims + 3 * count);
     const int E = dtype == OPENFFT_C2C_F32 ? 8 : 16;
     const int ext = dtype == OPENFFT_C2C_F32 ? FMT_C64 : FMT_C128;
@@ -276,17 +111,36 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
     const int twf = dtype == OPENFFT_C2C_F32 ? FMT_C64 : FMT_DF;
     std::vector<StageArgs> st((size_t)2 * 3 * count);
     cudaError_t e;
-    // twiddle tables per distinct length
-    std::vector<int> tw_len;
-    auto twiddle_for = [&](int n) -> const void* {
-        for (size_t k = 0; k < tw_len.size(); ++k) if (tw_len[k] == n) return b->twiddles[k];
-        void* t = nullptr;
-        if (dev_malloc((void**)&t, twiddle_bytes(n, twf))) return nullptr;
-        if (launch_twiddles(n, twf, t, nullptr)) { cudaFree(t); return nullptr; }
-        tw_len.push_back(n);
-        b->twiddles.push_back(t);
-        return t;
+    const bool f32 = dtype == OPENFFT_C2C_F32;
+    // twiddle table and radix plan per distinct length
+    std::vector<int> lens;
+    std::vector<MixPlan> plans;
+    auto tables_for = [&](int n, StageArgs& a) -> int {
+        size_t k = 0;
+        while (k < lens.size() && lens[k] != n) ++k;
+        if (k == lens.size()) {
+            const MixPlan pl = n <= kMaxLen ? mix_radix_plan(n, !f32) : MixPlan{};
+            if (pl.npass == 0) return fail(OPENFFT_ERR_UNSUPPORTED_RADIX, "axis length must factor into 2, 3, 5, 7 and be <= 2048");
+            void* t = nullptr;
+            if (dev_malloc((void**)&t, twiddle_bytes(n, twf))) { cudaGetLastError(); return fail(OPENFFT_ERR_NOMEM, "twiddle tables"); }
+            b->twiddles.push_back(t);
+            if (launch_twiddles(n, twf, t, nullptr)) { cudaGetLastError(); return fail(OPENFFT_ERR_NOMEM, "twiddle tables"); }
+            lens.push_back(n);
+            plans.push_back(pl);
+        }
+        a.tw = b->twiddles[k];
+        a.aux = reinterpret_cast<const void*>(k);        // its plan's index until the table has an address
+        return OPENFFT_OK;
     };
+    // Lines per tile: 8 while an SM holds three CTAs of such tiles of the longest axis,
+    // else the fewest (4 in FP32, 2 in double-float, which fit every length).
+    const size_t tables = sizeof(int64_t) * (size_t)(3 * count + 1) + sizeof(unsigned) * (size_t)(3 * count);
+    int nmax = 1;
+    for (int i = 0; i < 3 * count; ++i) nmax = dims[i] > nmax && dims[i] <= kMaxLen ? dims[i] : nmax;
+    b->G = f32 ? 4 : 2;
+    for (int G : {8, 4})
+        if (((tile_bytes_of(f32, G, nmax) + 15) & ~(size_t)15) + tables <= 75 * 1024) { b->G = G; break; }
+    b->smem = (tile_bytes_of(f32, b->G, nmax) + 15) & ~(size_t)15;
     for (int i = 0; i < count; ++i) {
         const int64_t Na = dims[3 * i], Nb = dims[3 * i + 1], Nc = dims[3 * i + 2];
         if (Na < 1 || Nb < 1 || Nc < 1 || P[i] < 1) { free_batch(b); return fail(OPENFFT_ERR_INVALID_ARG, "sizes and P must be >= 1"); }
@@ -312,27 +166,21 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
                 StageArgs& a = st[(size_t)dir * 3 * count + (size_t)s * count + i];
                 std::memset(&a, 0, sizeof(a));
                 const int n = (int)g.n;
-                if (n > kMaxLen || !radix_plan(n, a)) { free_batch(b); return fail(OPENFFT_ERR_UNSUPPORTED_RADIX, "axis length must factor into 2, 3, 5, 7 and be <= 2048"); }
-                int G = b->G;
                 const int64_t Mg = g.g2 ? g.M2 : g.M1;
-                while (G > 1 && (int64_t)(G / 2) >= Mg) G /= 2;
-                while (G > 1 && 2 * (size_t)n * (G + 1) * E > 200 * 1024) G /= 2;
-                // the tile bodies are compiled for the plan's G: other widths take the generic body
-                a.tw = twiddle_for(n);
-                if (!a.tw) { cudaGetLastError(); free_batch(b); return fail(OPENFFT_ERR_NOMEM, "twiddle tables"); }
+                const int G = b->G;
+                if (const int status = tables_for(n, a)) { free_batch(b); return status; }
                 a.M1 = g.M1; a.M2 = g.M2; a.S1 = g.S1; a.S2 = g.S2; a.Sk = g.Sk;
                 a.ngroups = (Mg + G - 1) / G;
                 a.scale = g.scale;
-                a.n = n; a.G = G; a.log2G = lg2(G);
+                a.n = n; a.G = G;
                 a.group_i2 = g.g2; a.contig_store = g.contig;
                 a.conj_in = g.cin; a.conj_out = g.cout; a.do_fft = 1;
                 a.in_fmt = g.in_fmt; a.out_fmt = g.out_fmt;
-                const size_t sm = 2 * (size_t)n * (G + 1) * E;
-                if (sm > b->smem) b->smem = sm;
             }
     }
     b->ctr_bytes = sizeof(BatchCounters) + sizeof(unsigned) * (size_t)3 * count;
-    if (dev_malloc((void**)&b->d_stages, st.size() * sizeof(StageArgs)) ||
+    const size_t stage_bytes = st.size() * sizeof(StageArgs), plan_bytes = plans.size() * sizeof(MixPlan);
+    if (dev_malloc((void**)&b->d_stages, stage_bytes + plan_bytes) ||
         dev_malloc((void**)&b->d_item_base, sizeof(int64_t) * (size_t)(2 * (3 * count + 1))) ||
         dev_malloc((void**)&b->d_need, sizeof(unsigned) * (size_t)(2 * 3 * count)) ||
         dev_malloc((void**)&b->d_ptrs, sizeof(void*) * (size_t)(2 * count)) ||
@@ -343,6 +191,18 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
         free_batch(b);
         return fail(OPENFFT_ERR_NOMEM, "batched plan tables");
     }
+    // launch shape: persistent, as many CTAs as fit (tile buffer + queue tables)
+    if (b->smem + tables > 200 * 1024) { free_batch(b); return fail(OPENFFT_ERR_UNSUPPORTED, "batch too large for the queue tables in shared memory"); }
+    int per_sm = 1;
+    e = persistent_ctas_per_sm(kernel_of(f32, b->G), kBatchThreads, b->smem + tables, &per_sm);
+    if (e) { free_batch(b); return fail(OPENFFT_ERR_CUDA, cudaGetErrorString(e)); }
+    b->grid = sms * (per_sm > 0 ? per_sm : 1);
+    {
+        int64_t tiles = 0;                       // of one direction's three stages
+        for (int q = 0; q < 3 * count; ++q) tiles += st[q].ngroups * (st[q].group_i2 ? st[q].M1 : st[q].M2);
+        const int64_t per = tiles / 3 / ((int64_t)b->grid * kItemsPerCta);
+        b->tiles_per_item = (int)(per < 1 ? 1 : (per > kMaxTilesPerItem ? kMaxTilesPerItem : per));
+    }
     // per direction (the two traverse the axes in opposite orders): tiles per
     // (stage, transform) and the stage-major queue prefix
     std::vector<int64_t> bases((size_t)2 * (3 * count + 1));
@@ -352,7 +212,7 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
         for (int q = 0; q < 3 * count; ++q) {
             const StageArgs& a = st[(size_t)dir * 3 * count + q];
             const int64_t tiles = a.ngroups * (a.group_i2 ? a.M1 : a.M2);
-            const int64_t items = (tiles + kTilesPerItem - 1) / kTilesPerItem;
+            const int64_t items = (tiles + b->tiles_per_item - 1) / b->tiles_per_item;
             bases[(size_t)dir * (3 * count + 1) + q] = acc;
             needs[(size_t)dir * 3 * count + q] = (unsigned)items;
             acc += items;
@@ -360,7 +220,13 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
         }
         bases[(size_t)dir * (3 * count + 1) + 3 * count] = acc;
     }
-    e = cudaMemcpy(b->d_stages, st.data(), st.size() * sizeof(StageArgs), cudaMemcpyHostToDevice);
+    // the stage descriptors, then the radix plans they point to
+    std::vector<unsigned char> up(stage_bytes + plan_bytes);
+    const MixPlan* d_plans = reinterpret_cast<const MixPlan*>(reinterpret_cast<unsigned char*>(b->d_stages) + stage_bytes);
+    for (StageArgs& a : st) a.aux = d_plans + reinterpret_cast<size_t>(a.aux);
+    std::memcpy(up.data(), st.data(), stage_bytes);
+    std::memcpy(up.data() + stage_bytes, plans.data(), plan_bytes);
+    e = cudaMemcpy(b->d_stages, up.data(), up.size(), cudaMemcpyHostToDevice);
     if (!e) e = cudaMemcpy(b->d_item_base, bases.data(), bases.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
     if (!e) e = cudaMemcpy(b->d_need, needs.data(), needs.size() * sizeof(unsigned), cudaMemcpyHostToDevice);
     if (!e) e = cudaMemcpy(b->d_scratch, b->scratch.data(), sizeof(void*) * (size_t)count, cudaMemcpyHostToDevice);
@@ -368,17 +234,6 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
     if (!e) e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming);
     if (!e) e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming);
     if (e) { free_batch(b); return fail(OPENFFT_ERR_CUDA, cudaGetErrorString(e)); }
-    // launch shape: persistent, as many CTAs as fit (tile buffer + queue tables)
-    b->smem = (b->smem + 15) & ~(size_t)15;
-    const size_t tables = sizeof(int64_t) * (size_t)(3 * count + 1) + sizeof(unsigned) * (size_t)(3 * count);
-    if (b->smem + tables > 200 * 1024) { free_batch(b); return fail(OPENFFT_ERR_UNSUPPORTED, "batch too large for the queue tables in shared memory"); }
-    int per_sm = 1;
-    if (b->arith == ARITH_F32)
-        e = persistent_ctas_per_sm((const void*)batch_kernel<ArF32, 16>, kBatchThreads, b->smem + tables, &per_sm);
-    else
-        e = persistent_ctas_per_sm((const void*)batch_kernel<ArDF, 8>, kBatchThreads, b->smem + tables, &per_sm);
-    if (e) { free_batch(b); return fail(OPENFFT_ERR_CUDA, cudaGetErrorString(e)); }
-    b->grid = sms * (per_sm > 0 ? per_sm : 1);
     e = cudaDeviceSynchronize();
     if (e) { free_batch(b); return fail(OPENFFT_ERR_CUDA, cudaGetErrorString(e)); }
     *out = b;
@@ -396,6 +251,7 @@ static cudaError_t launch_batch(BatchPlan* b, int dir_index, cudaStream_t s)
     d.ctr = reinterpret_cast<BatchCounters*>(b->d_ctr);
     d.done = reinterpret_cast<unsigned*>(b->d_ctr + sizeof(BatchCounters));
     d.count = b->count;
+    d.tiles_per_item = b->tiles_per_item;
     d.dir_index = dir_index;
     d.wait_budget = b->wait_budget;
     cudaError_t e = cudaMemsetAsync(b->d_ctr, 0, b->ctr_bytes, s);
@@ -404,9 +260,8 @@ static cudaError_t launch_batch(BatchPlan* b, int dir_index, cudaStream_t s)
     if (e) return e;
     const size_t tables = sizeof(int64_t) * (size_t)(3 * b->count + 1) + sizeof(unsigned) * (size_t)(3 * b->count);
     const size_t sm = b->smem + tables;
-    if (b->arith == ARITH_F32) batch_kernel<ArF32, 16><<<b->grid, kBatchThreads, sm, s>>>(d, b->smem);
-    else batch_kernel<ArDF, 8><<<b->grid, kBatchThreads, sm, s>>>(d, b->smem);
-    return cudaGetLastError();
+    void* args[] = {&d, &b->smem};
+    return cudaLaunchKernel(kernel_of(b->arith == ARITH_F32, b->G), dim3((unsigned)b->grid), dim3(kBatchThreads), args, sm, s);
 }
 
 int batch_exec(BatchPlan* b, const void* const* in, void* const* out, int dir, cudaStream_t user,

@@ -170,6 +170,9 @@ struct Mix {
                                                     const C* src, C* dst, const C* tw, int g, int slot, int slots)
     {
         switch (ps.radix) {
+        case 1:
+            if constexpr (FIRST) pass<1, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots);     // lines of one point
+            break;
         case 2: pass<2, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
         case 3: pass<3, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
         case 4: pass<4, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
@@ -192,28 +195,26 @@ struct Mix {
     }
 };
 
-template <class A, int G, bool REPEAT>
-__global__ void __launch_bounds__(kMixMaxThreads, mix_min_ctas())
-fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t ntiles)
+// Tiles tile, tile + step, ... below end of a stage, by a CTA of T threads.  cur and
+// oth: two tile buffers of G ld elements; tw: n elements for the length's twiddle
+// table, copied in here.  before_last() is called when the CTA begins its last tile.
+// Returns with the CTA's threads still reading the buffers.
+template <class A, int G, bool REPEAT, class BeforeLast>
+__device__ __forceinline__ void mix_run(const StageArgs& p, const MixPlan& plan, int64_t tile, int64_t step, int64_t end,
+                                        typename A::C* cur, typename A::C* oth, typename A::C* tw, int ld, int slots, int T,
+                                        BeforeLast before_last)
 {
     using M = Mix<A, G>;
     using C = typename A::C;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int ld = M::pitch(p.n);
-    C* cur = reinterpret_cast<C*>(smem_raw);
-    C* oth = cur + G * ld;
-    C* tw = oth + G * ld;
-    const int tid = threadIdx.x, T = blockDim.x;
-    const int g = M::line_of(tid), slot = M::slot_of(tid), slots = plan.slots, at = g * ld;
-    int64_t tile = blockIdx.x;
-    TileGeom tg = tile_geom<REPEAT>(p, tile, G);                // the grid has at most ntiles CTAs
-    grid_wait();
+    const int tid = threadIdx.x;
+    const int g = M::line_of(tid), slot = M::slot_of(tid), at = g * ld;
+    TileGeom tg = tile_geom<REPEAT>(p, tile, G);
     for (int i = tid; i < p.n; i += T) cp_async<M::E>(tw + i, reinterpret_cast<const C*>(p.tw) + i);
     M::issue_load(p, tg.line0, tg.lstride, tg.valid, cur, ld, tid, T);
-    for (; tile < ntiles; tile += gridDim.x) {
-        const int64_t next = tile + gridDim.x;
-        const TileGeom tn = tile_geom<REPEAT>(p, next < ntiles ? next : tile, G);
-        if (next >= ntiles) grid_release();
+    for (; tile < end; tile += step) {
+        const int64_t next = tile + step;
+        const TileGeom tn = tile_geom<REPEAT>(p, next < end ? next : tile, G);
+        if (next >= end) before_last();
         const bool mine = g < tg.valid;
         cp_async_wait_all();
         __syncthreads();
@@ -227,10 +228,10 @@ fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t 
                 __syncthreads();
             }
             // every thread has read `cur`: it takes the next tile while the last pass runs
-            if (next < ntiles) M::issue_load(p, tn.line0, tn.lstride, tn.valid, cur, ld, tid, T);
+            if (next < end) M::issue_load(p, tn.line0, tn.lstride, tn.valid, cur, ld, tid, T);
             if (mine) M::template dispatch<false>(p, plan.pass[np - 1], true, tg, oth + at, cur + at, tw, g, slot, slots);
         } else {
-            if (next < ntiles) M::issue_load(p, tn.line0, tn.lstride, tn.valid, oth, ld, tid, T);
+            if (next < end) M::issue_load(p, tn.line0, tn.lstride, tn.valid, oth, ld, tid, T);
             if (mine) M::template dispatch<true>(p, plan.pass[0], true, tg, cur + at, oth + at, tw, g, slot, slots);
             C* t = cur; cur = oth; oth = t;
         }
@@ -238,5 +239,23 @@ fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t 
     }
     cp_async_wait_all();
 }
+
+template <class A, int G, bool REPEAT>
+__global__ void __launch_bounds__(kMixMaxThreads, mix_min_ctas())
+fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t ntiles)
+{
+    using C = typename A::C;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int ld = Mix<A, G>::pitch(p.n);
+    C* buf = reinterpret_cast<C*>(smem_raw);
+    grid_wait();
+    // the grid has at most ntiles CTAs
+    mix_run<A, G, REPEAT>(p, plan, blockIdx.x, gridDim.x, ntiles, buf, buf + G * ld, buf + 2 * G * ld, ld, plan.slots,
+                          blockDim.x, [] { grid_release(); });
+}
+
+// The radix plan of length n for a policy of 16-byte (double-float) or 8-byte (FP32)
+// elements; npass = 0 if there is none.  pass[].radix etc. as the kernels read them.
+MixPlan mix_radix_plan(int n, bool df);
 
 }  // namespace ofg

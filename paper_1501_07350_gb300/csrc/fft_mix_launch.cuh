@@ -1,0 +1,87 @@
+// fft_mix_launch.cuh -- launch rule of the stage kernel of fft_mix.cuh.
+#pragma once
+#include <algorithm>
+#include <atomic>
+
+#include "fft_mix.cuh"
+
+namespace ofg {
+
+// What a launch on lines of one length needs.
+struct MixLaunch {
+    MixPlan plan;               // npass = 0: no launch
+    int threads, per_sm;
+    size_t smem;
+};
+
+// CTAs of 128 threads, or of 256 or 512 where an SM would hold fewer than 512
+// threads, and no more than the passes have butterflies for.  Sweeps of every count
+// on cubes of 36..448 points put 128 threads first or within 3 % almost
+// everywhere: 320^3 complex64 330 us, 350 with 64 or 192; 448^3 complex128
+// 3404 us with 256 (three CTAs per SM), 3561 with 128.
+template <class A, int G>
+MixLaunch make_launch(int n)
+{
+    MixLaunch l;
+    l.plan = mix_radix_plan(n, sizeof(typename A::C) >= 16);
+    l.smem = (2 * (size_t)G * Mix<A, G>::pitch(n) + n) * sizeof(typename A::C);
+    l.threads = l.per_sm = 0;
+    if (l.smem > 200 * 1024) l.plan.npass = 0;
+    if (l.plan.npass == 0) return l;
+    int nbf = 1;
+    for (int p = 0; p < l.plan.npass; ++p) nbf = std::max(nbf, l.plan.pass[p].nbf);
+    const int smem_ctas = (int)(227 * 1024 / (l.smem + 1024));
+    int T = 128;
+    while (T < kMixMaxThreads && smem_ctas * T < 512) T *= 2;
+    T = std::min(T, (G * nbf + 31) / 32 * 32);
+    l.threads = T;
+    l.plan.slots = T / G;
+    l.per_sm = std::min({32, 65536 / (64 * T), smem_ctas});
+    return l;
+}
+
+// Each length's launch is made on its first use and kept (at most kMaxLen of them
+// per arithmetic and tile width); two threads may both make one, and one is kept.
+template <class A, int G>
+const MixLaunch& mix_launch(int n)
+{
+    static std::atomic<const MixLaunch*> made[kMaxLen + 1] = {};
+    const MixLaunch* l = made[n].load(std::memory_order_acquire);
+    if (l) return *l;
+    const MixLaunch* mine = new MixLaunch(make_launch<A, G>(n));
+    if (made[n].compare_exchange_strong(l, mine, std::memory_order_acq_rel)) return *mine;
+    delete mine;
+    return *l;
+}
+
+template <class A, int G, bool REPEAT>
+cudaError_t launch_mix_r(const StageLaunch& L, cudaStream_t st, bool* handled)
+{
+    const MixLaunch& ml = mix_launch<A, G>(L.args.n);
+    if (ml.plan.npass == 0) return cudaSuccess;
+    auto kern = fft_mix_kernel<A, G, REPEAT>;
+    static int cached[kMaxDevices] = {};          // 1 once the kernel's attributes are set on the device
+    int* slot = device_slot(cached);
+    if (!slot || !*slot) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        if (!e) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        if (e) return e;
+        if (slot) *slot = 1;
+    }
+    StageArgs a = L.args;
+    const int64_t Mg = a.group_i2 ? a.M2 : a.M1;
+    a.ngroups = (Mg + G - 1) / G;
+    const int64_t ntiles = a.ngroups * (a.group_i2 ? a.M1 : a.M2) * (REPEAT ? a.M3 : 1);
+    if (ntiles > 0x7fffffffLL) return cudaSuccess;      // tiles are counted in 32 bits
+    *handled = true;
+    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)L.sms * ml.per_sm, ntiles));
+    return launch_chained(kern, (unsigned)grid, ml.threads, ml.smem, st, a, ml.plan, ntiles);
+}
+
+template <class A, int G>
+cudaError_t launch_mix_g(const StageLaunch& L, cudaStream_t st, bool* handled)
+{
+    return L.args.M3 > 1 ? launch_mix_r<A, G, true>(L, st, handled) : launch_mix_r<A, G, false>(L, st, handled);
+}
+
+}  // namespace ofg

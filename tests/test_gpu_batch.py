@@ -120,3 +120,17 @@ def test_batch_argument_errors(torch):
             of.openfft_exec_c2c(plan, x, torch.zeros_like(x), of.FORWARD)
     finally:
         of.openfft_destroy(plan)
+
+
+@pytest.mark.parametrize("dtype,tol", [(of.C2C_F32, 1e-5), (of.C2C_F64, 1e-12)])
+@pytest.mark.parametrize("shapes", [[(2048, 2, 3), (5, 4, 3)],           # the longest axis: the narrowest tiles
+                                    [(448, 6, 10), (12, 500, 9)],        # tiles of 4 lines in double-float
+                                    [(16, 16, 16)] * 40])                # more items than CTAs take at once, one tile each
+def test_batch_tile_widths(torch, shapes, dtype, tol):
+    Ps = [1] * len(shapes)
+    plan = of.openfft_plan_many(shapes, Ps, dtype)
+    try:
+        xs, xd = _inputs(torch, shapes, 99, dtype)
+        _check_batch(torch, plan, shapes, Ps, xs, xd, dtype, tol)
+    finally:
+        of.openfft_destroy(plan)
