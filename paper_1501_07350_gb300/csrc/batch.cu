@@ -172,6 +172,7 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
                 a.M1 = g.M1; a.M2 = g.M2; a.S1 = g.S1; a.S2 = g.S2; a.Sk = g.Sk;
                 a.ngroups = (Mg + G - 1) / G;
                 a.scale = g.scale;
+                split_scale(a);
                 a.n = n; a.G = G;
                 a.group_i2 = g.g2; a.contig_store = g.contig;
                 a.conj_in = g.cin; a.conj_out = g.cout; a.do_fft = 1;

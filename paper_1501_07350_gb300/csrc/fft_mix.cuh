@@ -110,7 +110,7 @@ struct Mix {
         char* ptr = reinterpret_cast<char*>(p.out) + o * EB;
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-            if (in_bounds(p.chk, o + q * step, p.out_elems)) put<A, CONJ_SCALE, EXT>(ptr, v[q], p.scale);
+            if (in_bounds(p.chk, o + q * step, p.out_elems)) put<A, CONJ_SCALE, EXT>(ptr, v[q], p);
             ptr += step * EB;
         }
     }

@@ -157,6 +157,7 @@ cudaError_t launch_stage(const StageLaunch& L0, cudaStream_t st)
 {
     StageLaunch L = L0;
     const int64_t elems = L.args.M1 * L.args.M2 * (L.args.M3 > 1 ? L.args.M3 : 1) * (int64_t)L.args.n;
+    split_scale(L.args);
     if (!L.args.in_elems) L.args.in_elems = elems;
     if (!L.args.out_elems) L.args.out_elems = elems;
     if (!L.args.chk) L.args.chk = L.status ? L.status : fallback_status_word();

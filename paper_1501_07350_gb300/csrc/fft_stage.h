@@ -32,6 +32,7 @@ struct StageArgs {
     int64_t M3, S3;
     int64_t ngroups;           // ceil(M_grouped / G)
     double scale;              // applied at store (1.0 = none)
+    float scale_hi, scale_lo;  // the same as an FP32 pair (split_scale)
     int n, G, log2G;
     int group_i2, contig_store;
     int npass;
@@ -45,6 +46,16 @@ struct StageArgs {
     int* chk;
 };
 
+
+// A positive output factor as an FP32 pair with hi + lo = scale: hi does not exceed
+// it and lo is positive, so that v hi + v lo of an infinite v is infinite.  Split
+// here and not by every thread (64x48x100 complex64 backward, three stages:
+// 13.2 -> 12.3 us).
+inline void split_scale(StageArgs& a)
+{
+    a.scale_hi = (float)(a.scale * (1.0 - 0x1p-24));
+    a.scale_lo = (float)(a.scale - (double)a.scale_hi);
+}
 
 struct StageLaunch {
     StageArgs args;

@@ -213,15 +213,14 @@ __device__ __forceinline__ void tile_fix(typename A::C* buf, int tid)
 }
 
 template <class A, bool CONJ_SCALE, bool EXT>
-__device__ __forceinline__ void put(void* ptr, typename A::C v, double scale)
+__device__ __forceinline__ void put(void* ptr, typename A::C v, const StageArgs& p)
 {
     if constexpr (CONJ_SCALE && std::is_same<A, ArF32>::value) {
         // the rounding of 1 / N is common to all outputs: undo it (80^3 backward
         // 1.58e-7 -> 1.47e-7 relative error)
-        const float kh = (float)scale, kl = (float)(scale - (double)kh);
-        v = make_float2(fmaf(v.x, kh, v.x * kl), -fmaf(v.y, kh, v.y * kl));
+        v = make_float2(fmaf(v.x, p.scale_hi, v.x * p.scale_lo), -fmaf(v.y, p.scale_hi, v.y * p.scale_lo));
     } else if constexpr (CONJ_SCALE) {
-        v = A::scale(A::conj(v), scale);
+        v = A::scale(A::conj(v), p.scale);
     }
     if constexpr (EXT) Io<A>::store_ext(ptr, v);
     else Io<A>::store_mid(ptr, v);
@@ -248,7 +247,7 @@ __device__ __forceinline__ void tile_store(const StageArgs& p, const TileGeom& t
 #pragma unroll 4
         for (int k = slot; k < N; k += T / G) {
             if (in_bounds(p.chk, tg.obase + g * tg.ostride + (int64_t)k * p.Sk, p.out_elems))
-                put<A, CONJ_SCALE, EXT>(ptr, buf[k * (G + 1) + g], p.scale);
+                put<A, CONJ_SCALE, EXT>(ptr, buf[k * (G + 1) + g], p);
             ptr += step;
         }
     } else {
@@ -257,7 +256,7 @@ __device__ __forceinline__ void tile_store(const StageArgs& p, const TileGeom& t
         for (int it = 0; it < ITERS; ++it) {
             const int e = tid + it * T;
             if ((TOTAL % T == 0 || e < TOTAL) && e / N < tg.valid && in_bounds(p.chk, tg.obase + e, p.out_elems))
-                put<A, CONJ_SCALE, EXT>(first + (int64_t)e * EB, buf[slot_of<N, G>(e)], p.scale);
+                put<A, CONJ_SCALE, EXT>(first + (int64_t)e * EB, buf[slot_of<N, G>(e)], p);
         }
     }
 }

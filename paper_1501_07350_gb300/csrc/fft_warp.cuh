@@ -167,7 +167,7 @@ __device__ __forceinline__ void warp_tile_store(const StageArgs& p, const TileGe
 #pragma unroll 4
         for (int k = slot; k < N; k += SL) {
             if (in_bounds(p.chk, tg.obase + g * tg.ostride + (int64_t)k * p.Sk, p.out_elems))
-                put<A, CONJ_SCALE, EXT>(ptr, line[wpad<CB>(k)], p.scale);
+                put<A, CONJ_SCALE, EXT>(ptr, line[wpad<CB>(k)], p);
             ptr += step;
         }
     } else {
@@ -183,7 +183,7 @@ __device__ __forceinline__ void warp_tile_store(const StageArgs& p, const TileGe
             for (int u = 0; u < (N + 31) / 32; ++u) {
                 const int k = lane + 32 * u;
                 if ((N % 32 == 0 || k < N) && in_bounds(p.chk, tg.obase + (int64_t)g * tg.ostride + k, p.out_elems))
-                    put<A, CONJ_SCALE, EXT>(ptr + k * EB, line[wpad<CB>(k)], p.scale);
+                    put<A, CONJ_SCALE, EXT>(ptr + k * EB, line[wpad<CB>(k)], p);
             }
         }
     }

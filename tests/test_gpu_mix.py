@@ -79,3 +79,17 @@ def test_complex64_arrays_at_8_byte_addresses(torch, shape):
                 assert oracle.rel_l2(yd.cpu().numpy().astype(np.complex128), ref) < TOL[of.C2C_F32]
     finally:
         of.openfft_destroy(plan)
+
+
+# The factor 1 / N is applied in two parts: a sum that overflows in the last butterfly of a
+# backward transform (the first value of a constant array, 4e38 before the factor) stays
+# infinite.  Powers of two (no second part) and other lengths (of either sign).
+@pytest.mark.parametrize("shape", [(64, 48, 100), (36, 10, 48), (256, 32, 32), (30, 28, 36), (9, 25, 14)])
+def test_overflow_stays_infinite(torch, shape):
+    n = int(np.prod(shape))
+    plan = of.openfft_plan(*shape, 1, of.C2C_F32)
+    try:
+        y = _exec(torch, plan, np.full(n, 4e38 / n, dtype=np.complex64), of.BACKWARD, of.C2C_F32)
+        assert y[0].real == np.inf, y[0]
+    finally:
+        of.openfft_destroy(plan)
