@@ -21,6 +21,8 @@
 // one buffer and writes global memory, so the next tile's copies (cp.async) go into
 // the other buffer while it runs.
 #pragma once
+#include <type_traits>
+
 #include "arith.cuh"
 #include "arith_pair.cuh"
 #include "fft_stage.h"
@@ -116,19 +118,27 @@ struct Mix {
     }
 
     // One pass from buffer src to buffer dst, or, the last one, to global memory.
-    template <int R, bool FIRST>
+    // The first pass takes its inputs from in(position) unless In is FromTile.
+    struct FromTile {
+        __device__ __forceinline__ C operator()(int) const { return A::zero(); }
+    };
+    template <int R, bool FIRST, class In>
     __device__ __forceinline__ static void pass(const StageArgs& p, const MixPass& ps, bool last, const TileGeom& tg,
-                                                const C* src, C* dst, const C* tw, int g, int slot, int slots)
+                                                const C* src, C* dst, const C* tw, int g, int slot, int slots, In in)
     {
+        constexpr bool kFromTile = std::is_same<In, FromTile>::value;
         // src, dst: this thread's line
         const int nbf = ps.nbf;
         for (int b = slot; b < nbf; b += slots) {
             C v[R];
             const C* x = src + b;
 #pragma unroll
-            for (int j = 0; j < R; ++j) v[j] = x[j * nbf];
+            for (int j = 0; j < R; ++j) {
+                if constexpr (kFromTile || !FIRST) v[j] = x[j * nbf];
+                else v[j] = in(b + j * nbf);
+            }
             int pos = b * R;                               // of the first result: t m R + k, b = t m + k
-            if constexpr (FIRST) {
+            if constexpr (FIRST && kFromTile) {
                 if constexpr (Io<A>::kConverts) {
                     if (p.in_fmt == FMT_C128) {
 #pragma unroll
@@ -139,7 +149,7 @@ struct Mix {
 #pragma unroll
                     for (int j = 0; j < R; ++j) v[j] = A::conj(v[j]);
                 }
-            } else {
+            } else if constexpr (!FIRST) {
                 const int t = (int)(((uint32_t)b * ps.inv) >> 20), k = b - t * ps.m;
                 pos = t * ps.m * R + k;
                 const int ks = k * ps.s;
@@ -165,29 +175,30 @@ struct Mix {
         }
     }
 
-    template <bool FIRST>
+    template <bool FIRST, class In = FromTile>
     __device__ __forceinline__ static void dispatch(const StageArgs& p, const MixPass& ps, bool last, const TileGeom& tg,
-                                                    const C* src, C* dst, const C* tw, int g, int slot, int slots)
+                                                    const C* src, C* dst, const C* tw, int g, int slot, int slots,
+                                                    In in = In())
     {
         switch (ps.radix) {
         case 1:
-            if constexpr (FIRST) pass<1, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots);     // lines of one point
+            if constexpr (FIRST) pass<1, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in);     // lines of one point
             break;
-        case 2: pass<2, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-        case 3: pass<3, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-        case 4: pass<4, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-        case 5: pass<5, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-        case 6: pass<6, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-        case 7: pass<7, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-        case 8: pass<8, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-        case 10: pass<10, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+        case 2: pass<2, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+        case 3: pass<3, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+        case 4: pass<4, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+        case 5: pass<5, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+        case 6: pass<6, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+        case 7: pass<7, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+        case 8: pass<8, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+        case 10: pass<10, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
         default:
             if constexpr (E == 8) {
                 switch (ps.radix) {
-                case 9: pass<9, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-                case 12: pass<12, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-                case 15: pass<15, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
-                default: pass<16, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots); break;
+                case 9: pass<9, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+                case 12: pass<12, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+                case 15: pass<15, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
+                default: pass<16, FIRST>(p, ps, last, tg, src, dst, tw, g, slot, slots, in); break;
                 }
             }
             break;

@@ -19,15 +19,11 @@ struct MixLaunch {
 // on cubes of 36..448 points put 128 threads first or within 3 % almost
 // everywhere: 320^3 complex64 330 us, 350 with 64 or 192; 448^3 complex128
 // 3404 us with 256 (three CTAs per SM), 3561 with 128.
-template <class A, int G>
-MixLaunch make_launch(int n)
+inline void size_launch(MixLaunch& l, int G)
 {
-    MixLaunch l;
-    l.plan = mix_radix_plan(n, sizeof(typename A::C) >= 16);
-    l.smem = (2 * (size_t)G * Mix<A, G>::pitch(n) + n) * sizeof(typename A::C);
     l.threads = l.per_sm = 0;
     if (l.smem > 200 * 1024) l.plan.npass = 0;
-    if (l.plan.npass == 0) return l;
+    if (l.plan.npass == 0) return;
     int nbf = 1;
     for (int p = 0; p < l.plan.npass; ++p) nbf = std::max(nbf, l.plan.pass[p].nbf);
     const int smem_ctas = (int)(227 * 1024 / (l.smem + 1024));
@@ -37,21 +33,46 @@ MixLaunch make_launch(int n)
     l.threads = T;
     l.plan.slots = T / G;
     l.per_sm = std::min({32, 65536 / (64 * T), smem_ctas});
+}
+
+template <class A, int G>
+MixLaunch make_launch(int n)
+{
+    MixLaunch l;
+    l.plan = mix_radix_plan(n, sizeof(typename A::C) >= 16);
+    l.smem = (2 * (size_t)G * Mix<A, G>::pitch(n) + n) * sizeof(typename A::C);
+    size_launch(l, G);
     return l;
 }
 
-// Each length's launch is made on its first use and kept (at most kMaxLen of them
-// per arithmetic and tile width); two threads may both make one, and one is kept.
+// The launch of length n that `make` makes, made on its first use and kept in `made`
+// (kMaxLen + 1 entries); two threads may both make one, and one is kept.
+template <class Make>
+const MixLaunch& kept_launch(std::atomic<const MixLaunch*>* made, int n, Make make)
+{
+    const MixLaunch* l = made[n].load(std::memory_order_acquire);
+    if (l) return *l;
+    const MixLaunch* mine = new MixLaunch(make(n));
+    if (made[n].compare_exchange_strong(l, mine, std::memory_order_acq_rel)) return *mine;
+    delete mine;
+    return *l;
+}
+
 template <class A, int G>
 const MixLaunch& mix_launch(int n)
 {
     static std::atomic<const MixLaunch*> made[kMaxLen + 1] = {};
-    const MixLaunch* l = made[n].load(std::memory_order_acquire);
-    if (l) return *l;
-    const MixLaunch* mine = new MixLaunch(make_launch<A, G>(n));
-    if (made[n].compare_exchange_strong(l, mine, std::memory_order_acq_rel)) return *mine;
-    delete mine;
-    return *l;
+    return kept_launch(made, n, make_launch<A, G>);
+}
+
+// A kernel's dynamic shared-memory limit and carveout, set once per device.
+inline cudaError_t prepare_kernel(const void* kern, int* slot)
+{
+    if (slot && *slot) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (!e) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (!e && slot) *slot = 1;
+    return e;
 }
 
 template <class A, int G, bool REPEAT>
@@ -61,13 +82,7 @@ cudaError_t launch_mix_r(const StageLaunch& L, cudaStream_t st, bool* handled)
     if (ml.plan.npass == 0) return cudaSuccess;
     auto kern = fft_mix_kernel<A, G, REPEAT>;
     static int cached[kMaxDevices] = {};          // 1 once the kernel's attributes are set on the device
-    int* slot = device_slot(cached);
-    if (!slot || !*slot) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (!e) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        if (e) return e;
-        if (slot) *slot = 1;
-    }
+    if (cudaError_t e = prepare_kernel((const void*)kern, device_slot(cached))) return e;
     StageArgs a = L.args;
     const int64_t Mg = a.group_i2 ? a.M2 : a.M1;
     a.ngroups = (Mg + G - 1) / G;

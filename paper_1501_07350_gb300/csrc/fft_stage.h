@@ -74,6 +74,8 @@ enum { KERNEL_AUTO = 0, KERNEL_WARP = 1, KERNEL_TILE = 2, KERNEL_GENERIC = 3 };
 // inverse's last stage; M1 = number of real lines, G = complex lines per CTA
 enum { KERNEL_R2C = 4, KERNEL_C2R = 5 };
 cudaError_t launch_real_stage(const StageLaunch& L, cudaStream_t st);
+// its any-length kernel (r2c_mix.cu); *handled = false when the stage has none
+cudaError_t launch_real_mix(const StageLaunch& L, cudaStream_t st, bool* handled);
 
 // Stage kernels are launched with programmatic stream serialisation: a stage's CTAs
 // may become resident while the stage before it drains, and wait there

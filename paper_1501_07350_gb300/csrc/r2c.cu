@@ -18,10 +18,11 @@
 //
 // Power-of-two n (32..512): one warp per complex line (a pair of real lines)
 // in the padded per-warp layout of the warp-per-line stage kernel, with its
-// radix passes; persistent CTAs of 8 warps.  Other n: one CTA per tile of 2G
-// real lines (G complex lines) in two ping-pong [n][G + 1] shared-memory
-// tiles, with the radix passes of the generic stage kernel (any supported n,
-// runtime radix plan).
+// radix passes; persistent CTAs of 8 warps.  Other n: the any-length kernel
+// (r2c_mix.cuh); on small arrays, where its tiles do not fit shared memory (about 1000
+// points) and for native FP64, one CTA per tile of 2G real lines (G complex lines) in
+// two ping-pong [n][G + 1] shared-memory tiles, with the radix passes of the generic
+// stage kernel (any supported n, runtime radix plan).
 #include <cuda_runtime.h>
 
 #include "fft_stage.h"
@@ -81,6 +82,20 @@ template <> struct RealPair<ArDF> {
         const float pl = __fmaf_rn(l, k.x, __fmaf_rn(h, k.y, __fmaf_rn(h, k.x, -ph)));
         return join_f64(ph, pl);
     }
+};
+
+// the packed policy (the warp kernels of power-of-two lengths): ArDF's bytes
+template <> struct RealPair<ArDP> {
+    using T = double;
+    using Scale = float2;
+    static constexpr bool kDF = true;
+    __device__ __forceinline__ static ArDP::C make(double a, double b) { return ArDP::from_float4(RealPair<ArDF>::make(a, b)); }
+    __device__ __forceinline__ static ArDP::C re_parts(ArDP::C u, ArDP::C v)
+    {
+        return ArDP::from_float4(RealPair<ArDF>::re_parts(ArDP::to_float4(u), ArDP::to_float4(v)));
+    }
+    __device__ __forceinline__ static Scale scale_of(double s) { return RealPair<ArDF>::scale_of(s); }
+    __device__ __forceinline__ static double part(ArDP::C z, int im, Scale k) { return RealPair<ArDF>::part(ArDP::to_float4(z), im, k); }
 };
 
 // i z, by exact sign changes: conj(-i conj z)
@@ -241,12 +256,23 @@ __device__ __forceinline__ void r2c_issue_raw(const T* __restrict__ x, int64_t L
     cp_async_commit();
 }
 
+// CTAs per SM the registers are shared among.  256-point double-float lines run
+// three of eight warps: 80 registers a thread hold the passes without spills
+// worth counting, and the third CTA covers the others' barriers (256^3 double:
+// 256.6 -> 246.8 us, inverse 247.4 -> 241.8; 64-point lines lose with three:
+// 64^3 inverse 15.1 -> 17.2).
+template <class C, int N>
+constexpr int real_min_blocks(int threads)
+{
+    return sizeof(C) >= 16 && N == 256 ? 3 : warp_min_blocks(threads, sizeof(C));
+}
+
 // Forward real stage, power-of-two N: warp w of tile t takes real lines
 // l0 + 2w and l0 + 2w + 1 (l0 = 2 G t); the CTA then separates the spectra of
 // its 2G lines and stores frequency k of all of them (2G consecutive
 // elements of the half array) at a time.
 template <class A, int N, int G>
-__global__ void __launch_bounds__(32 * G, warp_min_blocks(32 * G, sizeof(typename A::C)))
+__global__ void __launch_bounds__(32 * G, real_min_blocks<typename A::C, N>(32 * G))
 r2c_warp_kernel(const StageArgs p, int64_t ntiles)
 {
     using C = typename A::C;
@@ -259,7 +285,7 @@ r2c_warp_kernel(const StageArgs p, int64_t ntiles)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* tile = reinterpret_cast<C*>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const typename A::W* tw = reinterpret_cast<const typename A::W*>(p.tw);
+    const typename A::W* tw = A::table(p.tw, N);
     const T* x = reinterpret_cast<const T*>(p.in);
     const int64_t L = p.M1;
     C* line = tile + warp * LS;
@@ -340,7 +366,7 @@ __device__ __forceinline__ void c2r_issue_raw(const typename A::C* __restrict__ 
 // two half lines of the next tile into shared memory (cp.async) while the
 // current tile is transformed.
 template <class A, int N, int G>
-__global__ void __launch_bounds__(32 * G, warp_min_blocks(32 * G, sizeof(typename A::C)))
+__global__ void __launch_bounds__(32 * G, real_min_blocks<typename A::C, N>(32 * G))
 c2r_warp_kernel(const StageArgs p, int64_t ntiles)
 {
     using C = typename A::C;
@@ -352,7 +378,7 @@ c2r_warp_kernel(const StageArgs p, int64_t ntiles)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* tile = reinterpret_cast<C*>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const typename A::W* tw = reinterpret_cast<const typename A::W*>(p.tw);
+    const typename A::W* tw = A::table(p.tw, N);
     T* y = reinterpret_cast<T*>(p.out);
     const int64_t L = p.M1;
     C* line = tile + warp * LS;
@@ -431,15 +457,16 @@ cudaError_t launch_real_warp(const StageLaunch& L, cudaStream_t st)
                : launch_chained(c2r_warp_kernel<A, N, G>, (unsigned)grid, 32 * G, smem, st, L.args, ntiles);
 }
 
-template <class A>
+// AW: the policy of the warp kernels
+template <class A, class AW>
 cudaError_t launch_real_a(const StageLaunch& L, cudaStream_t st)
 {
     switch (L.args.n) {
-    case 32: return launch_real_warp<A, 32>(L, st);
-    case 64: return launch_real_warp<A, 64>(L, st);
-    case 128: return launch_real_warp<A, 128>(L, st);
-    case 256: return launch_real_warp<A, 256>(L, st);
-    case 512: return launch_real_warp<A, 512>(L, st);
+    case 32: return launch_real_warp<AW, 32>(L, st);
+    case 64: return launch_real_warp<AW, 64>(L, st);
+    case 128: return launch_real_warp<AW, 128>(L, st);
+    case 256: return launch_real_warp<AW, 256>(L, st);
+    case 512: return launch_real_warp<AW, 512>(L, st);
     default: break;
     }
     static int attr_r2c[kMaxDevices] = {}, attr_c2r[kMaxDevices] = {};     // attribute set on that device
@@ -469,10 +496,25 @@ cudaError_t launch_real_a(const StageLaunch& L, cudaStream_t st)
 
 cudaError_t launch_real_stage(const StageLaunch& L, cudaStream_t st)
 {
+    // The any-length kernel takes the lengths that are not powers of two, where the array
+    // has 2^15 points or more (240^3 transforms, generic kernel before: double 338 -> 310
+    // us, inverse 341 -> 315, float 111 -> 85, inverse 112 -> 89; 65536 lines of 9 points in
+    // double 38 -> 22, inverse 43 -> 39; 45^3 alike; on a smaller array its few CTAs take
+    // longer to a tile: 15^3 in float 10.2 against 13.9) and, in double-float, 128 (128^3
+    // 50.2 -> 47.3, inverse 51.4 -> 46.2) and 512 points (256x256x512 615 -> 559, inverse
+    // 637 -> 558).  The warp kernels are faster on the other powers of two (256^3 258 against
+    // 289, inverse 248 against 280; in float 97 against 99, inverse 95 against 117).
+    const int n = L.args.n;
+    const bool any = warp_length(n) ? L.arith == ARITH_DF && (n == 128 || n == 512) : L.args.M1 * n >= 32768;
+    if (any) {
+        bool handled = false;
+        cudaError_t e = launch_real_mix(L, st, &handled);
+        if (handled || e) return e;
+    }
     switch (L.arith) {
-    case ARITH_F64: return launch_real_a<ArF64>(L, st);
-    case ARITH_F32: return launch_real_a<ArF32>(L, st);
-    default: return launch_real_a<ArDF>(L, st);
+    case ARITH_F64: return launch_real_a<ArF64, ArF64>(L, st);
+    case ARITH_F32: return launch_real_a<ArF32, ArF32>(L, st);
+    default: return launch_real_a<ArDF, ArDP>(L, st);
     }
 }
 

@@ -156,3 +156,45 @@ def test_r2c_errors(torch):
     finally:
         of.openfft_destroy(rp)
         of.openfft_destroy(cp)
+
+
+# The any-length real stages: every radix in a first pass (where the inputs are formed),
+# odd lengths (no middle frequency, rows of every alignment), one- to many-pass plans,
+# an odd number of lines (ragged tiles, a line without a partner) and 2^15 points or just
+# more (the kernel's smallest array), tiles of 4 and 8 lines, arrays at the smallest
+# alignment of their type.
+@pytest.mark.parametrize("dtype", [of.R2C_F64, of.R2C_F32])
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 15, 18, 25, 30, 49, 75, 90, 100, 128, 144, 225, 240, 243,
+                               250, 343, 360, 450, 512, 625, 800])
+def test_any_length_real_stages(torch, n, dtype):
+    odd = sorted(3**a * 5**b * 7**c for a in range(7) for b in range(5) for c in range(4))
+    nb = next(m for m in odd if 21 * m * n >= 32768)
+    shape, nh = (21, nb, n), n // 2 + 1
+    lines = 21 * nb
+    tol = TOL[dtype]
+    rng = np.random.default_rng(n)
+    x = rng.standard_normal(shape)
+    rt, ct = _types(torch, dtype)
+    x = x.astype(np.float64 if dtype == of.R2C_F64 else np.float32).astype(np.float64)
+    ref = np.ascontiguousarray(np.fft.rfftn(x).transpose(2, 1, 0)).reshape(-1)
+    plan = of.openfft_plan(*shape, 1, dtype)
+    try:
+        y = _r2c(torch, plan, x, dtype, nh)
+        assert oracle.rel_l2(y, ref) < tol, n
+        z = _c2r(torch, plan, ref, dtype, x.size)
+        assert oracle.rel_l2(z, x.reshape(-1)) < tol, n
+        if n in (128, 512):                # the power-of-two float kernels want 16-byte addresses, as documented
+            return
+        # one element off the allocation's own alignment (complex128 stays on 16 bytes)
+        xd = torch.empty(x.size + 1, dtype=rt, device="cuda")[1:]
+        xd.copy_(torch.from_numpy(x.reshape(-1)))
+        yd = torch.full((nh * lines + 1,), float("nan"), dtype=ct, device="cuda")[1:]
+        of.openfft_exec_r2c(plan, xd, yd)
+        of.openfft_sync(plan)
+        assert oracle.rel_l2(yd.cpu().numpy().astype(np.complex128), ref) < tol, n
+        zd = torch.full((x.size + 1,), float("nan"), dtype=rt, device="cuda")[1:]
+        of.openfft_exec_c2r(plan, yd, zd)
+        of.openfft_sync(plan)
+        assert oracle.rel_l2(zd.cpu().numpy().astype(np.float64), x.reshape(-1)) < 2 * tol, n
+    finally:
+        of.openfft_destroy(plan)
