@@ -5,8 +5,7 @@
 // per-pass twiddle tables).  What differs is the output: the last radix pass
 // writes its results into a staging area laid out as the output needs them,
 // and one thread hands the whole tile to the tensor memory accelerator (a TMA
-// tensor store, or one bulk copy per line for contiguous output), which
-// drains it while the CTA goes on with the next tile.
+// tensor store, or one bulk copy for a line of contiguous output).
 // Transposed output (the fused transposes of steps (4)-(6), Sec. 3.1.1): the
 // tile's G lines are consecutive in the output at every frequency k, so the
 // staging area is [k][G lines] of 16-byte elements in the swizzle of the
@@ -16,13 +15,20 @@
 // line coordinate) with element strides (1, Sk, So).
 //
 // Tile layout: the tile's lines, which the staging area overlays once every
-// line's last-pass inputs are in registers (a CTA barrier); the next tile's
-// copies (cp.async) start when the copy engine has read the staging area.
-// The lines are the CTA's only shared memory (19 KB for 4 lines of 256
-// points, 38 KB for 4 of 512), so many CTAs stay resident (8 and 4 per SM,
-// 32 warps) and one CTA's loads overlap the others' passes.  Measured on
-// 256^3 this beat two input buffers with a separate staging area (4 CTAs per
-// SM) by 6 %; on 512^3 double buffering with 3 CTAs per SM was 9 % slower.
+// line's last-pass inputs are in registers (a CTA barrier).  They are the CTA's
+// only shared memory (19 KB for 4 lines of 256 points, 38 KB for 4 of 512), so 32
+// warps stay resident on an SM, and one CTA's loads overlap the others' passes:
+// double buffering held fewer CTAs and was 6-9 % slower.
+//
+// A CTA takes one tile and ends when the copy engine has read it, and the
+// hardware's scheduler starts the next one.  Persistent CTAs with a fixed share of
+// the tiles each had left the SMs with 24 of 32 warps on average: CTAs of an SM
+// advance at different rates, and those that finished early left their warps idle
+// (512^3 3740 -> 3290 us, 256^3 428 -> 381; persistent CTAs that claim tiles from the
+// scheduler, clusterlaunchcontrol, 3377 and 396).  For the same reason a stage of
+// contiguous output, whose lines share nothing, has a CTA per line (3290 -> 3220, 381 -> 375).
+// What bounds the kernel is the arithmetic: the FP32 pipe's packed operations and the
+// issue slots beside them.
 #pragma once
 #include <cuda.h>
 
@@ -47,8 +53,6 @@ __device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t byt
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // the copy engine has read every committed group's shared memory
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// every committed group is complete
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // make this thread's generic-proxy shared-memory writes visible to the copy engine
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // the passes of line g synchronise the WPL warps that share it: the warp
@@ -67,17 +71,10 @@ __device__ __forceinline__ void line_sync(int g)
 // has 32 radix-8 butterflies per pass, and a second warp would idle there.
 template <int N>
 constexpr int tma_wpl() { return N == 512 ? 2 : 1; }
-// CTAs per SM the register allocation is sized for: 64 registers a thread,
-// 32 warps per SM
-template <int N>
-constexpr int tma_min_ctas() { return N == 256 ? 8 : 4; }
-
 // byte offset of output element (frequency k, tile line g) in the transposed
-// staging area: the tensor store's swizzle for rows of G x 16 bytes
-template <int G>
+// staging area: the tensor store's swizzle for rows of 4 x 16 bytes
 __device__ __forceinline__ uint32_t staged_offset(int k, int g)
 {
-    static_assert(G == 4, "rows of 64 bytes");
     return (uint32_t)k * 64u + ((uint32_t)(g ^ ((k >> 1) & 3)) << 4);
 }
 
@@ -209,7 +206,7 @@ struct TmaLine {
 #pragma unroll
                 for (int q = 0; q < R; ++q) {
                     const int k = base + m * q;
-                    const uint32_t off = CONTIG ? (uint32_t)k * 16u : staged_offset<G>(k, g);
+                    const uint32_t off = CONTIG ? (uint32_t)k * 16u : staged_offset(k, g);
                     *reinterpret_cast<uint4*>(stage + off) = out16<CONJ_SCALE, EXT>(v[u][q], scale);
                 }
             }
@@ -239,74 +236,61 @@ __device__ __forceinline__ void tma_issue_load(const StageArgs& p, const TileGeo
 
 template <int N, int G>
 constexpr size_t tma_stage_bytes() { return (size_t)N * G * 16; }
-// 1024-byte alignment slack (the 128-byte swizzle), then the tile's lines,
-// which the staging area overlays
-template <int N, int G>
-constexpr size_t tma_smem_bytes() { return 1024 + (size_t)G * warp_line_stride<16>(N) * 16; }
+// the tile's lines, which the staging area overlays; for the tensor store's swizzle
+// that area starts on 1024 bytes
+template <int N, int G, bool CONTIG>
+constexpr size_t tma_smem_bytes() { return (CONTIG ? 0 : 1024) + (size_t)G * warp_line_stride<16>(N) * 16; }
 
 template <int N, int G, bool CONTIG, bool CONJ_SCALE, bool EXT>
-__global__ void __launch_bounds__(32 * G * tma_wpl<N>(), tma_min_ctas<N>())
-fft_warp_tma_kernel(const StageArgs p, int64_t ntiles, const __grid_constant__ CUtensorMap tmap)
+__global__ void __launch_bounds__(32 * G * tma_wpl<N>(), 32 / (G * tma_wpl<N>()))
+fft_warp_tma_kernel(const StageArgs p, const __grid_constant__ CUtensorMap tmap)
 {
     constexpr int WPL = tma_wpl<N>();
     using L = TmaLine<N, WPL>;
     using C = ArDP::C;
     constexpr int LS = L::LS;
     static_assert(tma_stage_bytes<N, G>() <= (size_t)G * LS * 16, "staging must fit the lines");
+    static_assert(G == (CONTIG ? 1 : 4), "a CTA per line of contiguous output; rows of 64 bytes");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint32_t base = smem_addr(smem_raw);
-    unsigned char* stage = smem_raw + (((base + 1023u) & ~1023u) - base);
-    C* const lines = reinterpret_cast<C*>(stage);
+    unsigned char* stage = smem_raw + (CONTIG ? 0u : ((base + 1023u) & ~1023u) - base);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = warp / WPL, w = warp % WPL;
-    C* const line = lines + g * LS;
+    C* const line = reinterpret_cast<C*>(stage) + g * LS;
     const ArDP::W* tw = ArDP::table(p.tw, N);
-    const bool convert = p.in_fmt == FMT_C128;
+    const int64_t tile = blockIdx.x;
+    const TileGeom tg = tile_geom(p, tile, G);
     grid_wait();
-
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const TileGeom tg = tile_geom(p, tile, G);
-        if (tile + gridDim.x >= ntiles) grid_release();
-        // the previous tile's store has read the staging area: copy this tile in
-        const bool leader = CONTIG ? (w == 0 && lane == 0) : tid == 0;
-        if (leader) bulk_wait_read_all();
-        if constexpr (CONTIG) line_sync<WPL>(g);
-        else __syncthreads();
-        tma_issue_load<N, WPL>(p, tg, g, line, lane, w);
-        cp_async_wait_all();
-        line_sync<WPL>(g);
-        if (convert) {
-            if (p.conj_in) L::template passes<0, 3>(line, tw, lane, w, g);
-            else L::template passes<0, 2>(line, tw, lane, w, g);
-        } else if (p.conj_in) {
-            L::template passes<0, 1>(line, tw, lane, w, g);
-        } else {
-            L::template passes<0, 0>(line, tw, lane, w, g);
-        }
-        L::template last_pass<G, CONTIG, CONJ_SCALE, EXT>(line, tw, CONTIG ? reinterpret_cast<unsigned char*>(line) : stage,
-                                                         lane, w, g, p.scale);
-        fence_proxy_async_smem();
+    grid_release();
+    tma_issue_load<N, WPL>(p, tg, g, line, lane, w);
+    cp_async_wait_all();
+    line_sync<WPL>(g);
+    if (p.in_fmt == FMT_C128) {
+        if (p.conj_in) L::template passes<0, 3>(line, tw, lane, w, g);
+        else L::template passes<0, 2>(line, tw, lane, w, g);
+    } else if (p.conj_in) {
+        L::template passes<0, 1>(line, tw, lane, w, g);
+    } else {
+        L::template passes<0, 0>(line, tw, lane, w, g);
+    }
+    L::template last_pass<G, CONTIG, CONJ_SCALE, EXT>(line, tw, CONTIG ? reinterpret_cast<unsigned char*>(line) : stage,
+                                                     lane, w, g, p.scale);
+    fence_proxy_async_smem();
+    if constexpr (CONTIG) line_sync<WPL>(g);
+    else __syncthreads();
+    if (tid == 0) {
         if constexpr (CONTIG) {
-            line_sync<WPL>(g);
-            if (leader && g < tg.valid) {
-                const int64_t o = tg.obase + g * tg.ostride;
-                if (in_bounds(p.chk, o, p.out_elems) && in_bounds(p.chk, o + N - 1, p.out_elems))
-                    bulk_store(reinterpret_cast<char*>(p.out) + o * 16, smem_addr(line), N * 16u);
-                bulk_commit();
-            }
-            continue;
-        }
-        __syncthreads();
-        if (tid == 0) {
+            if (in_bounds(p.chk, tg.obase, p.out_elems) && in_bounds(p.chk, tg.obase + N - 1, p.out_elems))
+                bulk_store(reinterpret_cast<char*>(p.out) + tg.obase * 16, smem_addr(line), N * 16u);
+        } else {
 #pragma unroll
             for (int kb = 0; kb < (N + 255) / 256; ++kb)
                 tma_store_3d(&tmap, smem_addr(stage) + (uint32_t)kb * 256u * (uint32_t)(G * 16),
                              (int)((tile % p.ngroups) * G * 4), kb * 256, (int)(tile / p.ngroups));
-            bulk_commit();
         }
+        bulk_commit();
+        bulk_wait_read_all();
     }
-    cp_async_wait_all();
-    if (CONTIG ? (tid % (32 * WPL)) == 0 : tid == 0) bulk_wait_all();
 }
 
 // host side ----------------------------------------------------------------
@@ -360,20 +344,16 @@ template <int N, int G, bool CONTIG, bool CONJ_SCALE, bool EXT>
 cudaError_t launch_warp_tma_v(const StageLaunch& L, const CUtensorMap& map, cudaStream_t st)
 {
     auto kern = fft_warp_tma_kernel<N, G, CONTIG, CONJ_SCALE, EXT>;
-    const size_t smem = tma_smem_bytes<N, G>();
-    static int cached[kMaxDevices] = {};
+    const size_t smem = tma_smem_bytes<N, G, CONTIG>();
+    static int cached[kMaxDevices] = {};          // 1 once the kernel's attributes are set on the device
     int* slot = device_slot(cached);
-    int per_sm = slot ? *slot : 0;
-    if (per_sm == 0) {
+    if (!slot || !*slot) {
+        int per_sm = 0;
         cudaError_t e = persistent_ctas_per_sm((const void*)kern, 32 * G * tma_wpl<N>(), smem, &per_sm);
         if (e) return e;
-        if (slot) *slot = per_sm;
+        if (slot) *slot = 1;
     }
-    const int64_t ntiles = L.grid;
-    int64_t grid = (int64_t)L.sms * per_sm;
-    if (grid > ntiles) grid = ntiles;
-    if (grid < 1) grid = 1;
-    return launch_chained(kern, (unsigned)grid, 32 * G * tma_wpl<N>(), smem, st, L.args, ntiles, map);
+    return launch_chained(kern, (unsigned)L.grid, 32 * G * tma_wpl<N>(), smem, st, L.args, map);
 }
 
 // The asynchronous-output kernel for n = 256 / 512 in tiles of G lines,
@@ -383,12 +363,16 @@ cudaError_t launch_warp_tma_n(const StageLaunch& L0, cudaStream_t st, bool* hand
 {
     StageLaunch L = L0;
     StageArgs& a = L.args;
-    a.G = G;
-    a.ngroups = ((a.group_i2 ? a.M2 : a.M1) + G - 1) / G;
+    const bool contig = a.contig_store != 0;
+    a.G = contig ? 1 : G;
+    a.ngroups = ((a.group_i2 ? a.M2 : a.M1) + a.G - 1) / a.G;
     L.grid = a.ngroups * (a.group_i2 ? a.M1 : a.M2);
+    if (L.grid < 1 || L.grid > 0x7fffffffLL) {
+        *handled = false;
+        return cudaSuccess;
+    }
     CUtensorMap map;
     std::memset(&map, 0, sizeof(map));
-    const bool contig = a.contig_store != 0;
     if (contig) {
         if (a.group_i2 || a.S1 != a.n || a.Sk != 1 || (reinterpret_cast<uintptr_t>(a.out) & 15) != 0) {
             *handled = false;
@@ -415,8 +399,8 @@ cudaError_t launch_warp_tma_n(const StageLaunch& L0, cudaStream_t st, bool* hand
     *handled = true;
     const bool ext = a.out_fmt != FMT_DF, cs = a.conj_out != 0;
     if (contig) {
-        if (cs) return ext ? launch_warp_tma_v<N, G, true, true, true>(L, map, st) : launch_warp_tma_v<N, G, true, true, false>(L, map, st);
-        return ext ? launch_warp_tma_v<N, G, true, false, true>(L, map, st) : launch_warp_tma_v<N, G, true, false, false>(L, map, st);
+        if (cs) return ext ? launch_warp_tma_v<N, 1, true, true, true>(L, map, st) : launch_warp_tma_v<N, 1, true, true, false>(L, map, st);
+        return ext ? launch_warp_tma_v<N, 1, true, false, true>(L, map, st) : launch_warp_tma_v<N, 1, true, false, false>(L, map, st);
     }
     if (cs) return ext ? launch_warp_tma_v<N, G, false, true, true>(L, map, st) : launch_warp_tma_v<N, G, false, true, false>(L, map, st);
     return ext ? launch_warp_tma_v<N, G, false, false, true>(L, map, st) : launch_warp_tma_v<N, G, false, false, false>(L, map, st);

@@ -1,11 +1,14 @@
 """Stages launched as a chain (a stage's CTAs may become resident while the stage
 before it drains): results of transforms enqueued back to back, on one stream, on two
 and replayed from a captured graph are bit for bit those of transforms run one at a
-time."""
+time.  And the stages with a CTA per tile, against the FP64 oracle (the bar of the other
+parity tests, relative L2 <= 1e-12)."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_1501_07350_gb300 import openfft as of
+from paper_1501_07350_gb300 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -73,3 +76,25 @@ def test_chained_transforms_match_single_ones(torch, shape, dtype):
     check()
     for p in plans:
         p.close()
+
+
+# 256- and 512-point double-float stages: one to two tiles (3, 5 lines), a ragged last tile
+# (126 lines), more tiles than an SM holds CTAs for; transposed and, as the last stage,
+# contiguous output (a CTA per line), entry and exit formats in each position.
+@pytest.mark.parametrize("n", [256, 512])
+@pytest.mark.parametrize("other", [(1, 3), (5, 1), (9, 14), (75, 98)])
+def test_a_cta_per_tile(torch, n, other):
+    a, b = other
+    for shape in ((n, a, b), (a, n, b), (a, b, n)):
+        x = synth.complex_field(shape, seed=n)
+        xd = torch.from_numpy(np.ascontiguousarray(x.reshape(-1))).to(device="cuda", dtype=torch.complex128)
+        plan = of.Plan(*shape, 1, of.C2C_F64)
+        try:
+            for direction, odir in ((of.FORWARD, oracle.FORWARD), (of.BACKWARD, oracle.BACKWARD)):
+                yd = torch.full_like(xd, float("nan"))
+                plan.exec(xd, yd, direction)
+                torch.cuda.synchronize()
+                err = oracle.rel_l2(yd.cpu().numpy(), oracle.fft3d(x, *shape, 1, odir))
+                assert err < 1e-12, (shape, direction, err)
+        finally:
+            plan.close()
