@@ -89,7 +89,7 @@ cudaError_t launch_mix_r(const StageLaunch& L, cudaStream_t st, bool* handled)
     const int64_t ntiles = a.ngroups * (a.group_i2 ? a.M1 : a.M2) * (REPEAT ? a.M3 : 1);
     if (ntiles > 0x7fffffffLL) return cudaSuccess;      // tiles are counted in 32 bits
     *handled = true;
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)L.sms * ml.per_sm, ntiles));
+    const int64_t grid = tile_grid<A>(ntiles, (int64_t)L.sms * ml.per_sm);
     return launch_chained(kern, (unsigned)grid, ml.threads, ml.smem, st, a, ml.plan, ntiles);
 }
 

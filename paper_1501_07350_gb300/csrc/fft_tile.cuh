@@ -212,6 +212,23 @@ __device__ __forceinline__ void tile_fix(typename A::C* buf, int tid)
     }
 }
 
+// Grid of a kernel whose CTAs take tiles grid, 2 grid, ... beyond their own, of which
+// `resident` fit on the device.  Double-float: eight times those.  With one share of
+// the tiles per resident CTA the SMs' warps idled towards the end (CTAs of an SM advance at
+// different rates), with a CTA per tile nothing is copied ahead: 240x288x320 complex128
+// takes 840 us with 1, 805 with 2, 785 with 4, 778 with 8 and 804 with a CTA per tile;
+// 384x384x192 991, 958, 925, 900; 512x128x256 429, 416, 411, 410, 406; 256^3 real forward
+// 227, 223, 220, 218, 218.  FP32 stages wait for memory more than for issue slots, and a
+// longer grid costs them copies ahead: 180x200x225 86.9 with 1 and 88.2 with 4 (512^3 1452
+// and 1407), so they keep one.
+struct ArDP;
+template <class A>
+inline int64_t tile_grid(int64_t ntiles, int64_t resident, int waves = 8)
+{
+    if (std::is_same<A, ArDP>::value) resident *= waves;
+    return ntiles < 1 ? 1 : (ntiles < resident ? ntiles : (resident < 1 ? 1 : resident));
+}
+
 template <class A, bool CONJ_SCALE, bool EXT>
 __device__ __forceinline__ void put(void* ptr, typename A::C v, const StageArgs& p)
 {

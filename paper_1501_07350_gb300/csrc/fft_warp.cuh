@@ -310,9 +310,7 @@ cudaError_t launch_warp_n(const StageLaunch& L, cudaStream_t st)
         if (slot) *slot = blocks_per_sm;
     }
     const int64_t ntiles = L.grid;
-    int64_t grid = (int64_t)L.sms * blocks_per_sm;
-    if (grid > ntiles) grid = ntiles;
-    if (grid < 1) grid = 1;
+    const int64_t grid = tile_grid<A>(ntiles, (int64_t)L.sms * blocks_per_sm);
     return launch_chained(fft_warp_kernel<A, N, G>, (unsigned)grid, T, smem, st, L.args, ntiles);
 }
 

@@ -450,9 +450,7 @@ cudaError_t launch_real_warp(const StageLaunch& L, cudaStream_t st)
         if (slot) *slot = per_sm;
     }
     const int64_t ntiles = (L.args.M1 + 2 * G - 1) / (2 * G);
-    int64_t grid = (int64_t)L.sms * per_sm;
-    if (grid > ntiles) grid = ntiles;
-    if (grid < 1) grid = 1;
+    const int64_t grid = tile_grid<A>(ntiles, (int64_t)L.sms * per_sm);
     return fwd ? launch_chained(r2c_warp_kernel<A, N, G>, (unsigned)grid, 32 * G, smem, st, L.args, ntiles)
                : launch_chained(c2r_warp_kernel<A, N, G>, (unsigned)grid, 32 * G, smem, st, L.args, ntiles);
 }

@@ -30,7 +30,8 @@ cudaError_t launch_real_g(const StageLaunch& L, cudaStream_t st, bool* handled)
     if (cudaError_t e = prepare_kernel(kern, device_slot(cached[fwd]))) return e;
     *handled = true;
     const int64_t ntiles = (L.args.M1 + 2 * G - 1) / (2 * G);
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)L.sms * ml.per_sm, ntiles));
+    // 180x200x225 double forward 200 us with one share a CTA, 195 with 4, 201 with 8
+    const unsigned grid = (unsigned)tile_grid<A>(ntiles, (int64_t)L.sms * ml.per_sm, 4);
     return fwd ? launch_chained(real_mix_kernel<A, G, true>, grid, ml.threads, ml.smem, st, L.args, ml.plan, ntiles)
                : launch_chained(real_mix_kernel<A, G, false>, grid, ml.threads, ml.smem, st, L.args, ml.plan, ntiles);
 }

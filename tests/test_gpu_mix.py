@@ -93,3 +93,17 @@ def test_overflow_stays_infinite(torch, shape):
         assert y[0].real == np.inf, y[0]
     finally:
         of.openfft_destroy(plan)
+
+
+# Double-float grids: as many CTAs as tiles (more than the SMs hold), and fewer (each CTA
+# takes several), in the same transform: 29160 to 45000 lines in tiles of 4.
+def test_grids_of_several_waves(torch):
+    shape = (250, 180, 162)
+    x = synth.complex_field(shape, seed=7)
+    plan = of.openfft_plan(*shape, 1, of.C2C_F64)
+    try:
+        for direction, odir in ((of.FORWARD, oracle.FORWARD), (of.BACKWARD, oracle.BACKWARD)):
+            err = oracle.rel_l2(_exec(torch, plan, x, direction, of.C2C_F64), oracle.fft3d(x, *shape, 1, odir))
+            assert err < TOL[of.C2C_F64], (direction, err)
+    finally:
+        of.openfft_destroy(plan)
