@@ -208,12 +208,10 @@ struct Mix {
 
 // Tiles tile, tile + step, ... below end of a stage, by a CTA of T threads.  cur and
 // oth: two tile buffers of G ld elements; tw: n elements for the length's twiddle
-// table, copied in here.  before_last() is called when the CTA begins its last tile.
-// Returns with the CTA's threads still reading the buffers.
-template <class A, int G, bool REPEAT, class BeforeLast>
+// table, copied in here.  Returns with the CTA's threads still reading the buffers.
+template <class A, int G, bool REPEAT>
 __device__ __forceinline__ void mix_run(const StageArgs& p, const MixPlan& plan, int64_t tile, int64_t step, int64_t end,
-                                        typename A::C* cur, typename A::C* oth, typename A::C* tw, int ld, int slots, int T,
-                                        BeforeLast before_last)
+                                        typename A::C* cur, typename A::C* oth, typename A::C* tw, int ld, int slots, int T)
 {
     using M = Mix<A, G>;
     using C = typename A::C;
@@ -225,7 +223,6 @@ __device__ __forceinline__ void mix_run(const StageArgs& p, const MixPlan& plan,
     for (; tile < end; tile += step) {
         const int64_t next = tile + step;
         const TileGeom tn = tile_geom<REPEAT>(p, next < end ? next : tile, G);
-        if (next >= end) before_last();
         const bool mine = g < tg.valid;
         cp_async_wait_all();
         __syncthreads();
@@ -262,7 +259,7 @@ fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t 
     grid_wait();
     // the grid has at most ntiles CTAs
     mix_run<A, G, REPEAT>(p, plan, blockIdx.x, gridDim.x, ntiles, buf, buf + G * ld, buf + 2 * G * ld, ld, plan.slots,
-                          blockDim.x, [] { grid_release(); });
+                          blockDim.x);
 }
 
 // The radix plan of length n for a policy of 16-byte (double-float) or 8-byte (FP32)

@@ -42,7 +42,6 @@ fft_stage_kernel(const StageArgs p)
     __shared__ int64_t s_in[kMaxLinesPerCta];
     __shared__ int64_t s_out[kMaxLinesPerCta];
     grid_wait();
-    grid_release();
     generic_stage_tile<A>(p, blockIdx.x, smem_raw, s_in, s_out);
 }
 

@@ -315,7 +315,6 @@ fft_tile_kernel(const StageArgs p, int64_t ntiles)
     if (tile < ntiles) tile_issue_loads<A, N, G, T>(p, tile_geom(p, tile, G), cur, tid);
     for (; tile < ntiles; tile += gridDim.x) {
         const TileGeom tg = tile_geom(p, tile, G);
-        if (tile + gridDim.x >= ntiles) grid_release();
         cp_async_wait_all();
         if (convert) { if (p.conj_in) tile_fix<A, N, G, T, true, true>(cur, tid); else tile_fix<A, N, G, T, true, false>(cur, tid); }
         else if (p.conj_in) tile_fix<A, N, G, T, false, true>(cur, tid);

@@ -266,7 +266,6 @@ fft_warp_kernel(const StageArgs p, int64_t ntiles)
     }
     for (; tile < ntiles; tile += gridDim.x) {
         const TileGeom tg = tile_geom(p, tile, G);
-        if (tile + gridDim.x >= ntiles) grid_release();
         C* line0 = cur + g0 * LS;
         if (!DB) {
 #pragma unroll

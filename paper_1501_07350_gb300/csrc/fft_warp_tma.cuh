@@ -261,7 +261,6 @@ fft_warp_tma_kernel(const StageArgs p, const __grid_constant__ CUtensorMap tmap)
     const int64_t tile = blockIdx.x;
     const TileGeom tg = tile_geom(p, tile, G);
     grid_wait();
-    grid_release();
     tma_issue_load<N, WPL>(p, tg, g, line, lane, w);
     cp_async_wait_all();
     line_sync<WPL>(g);
@@ -289,6 +288,7 @@ fft_warp_tma_kernel(const StageArgs p, const __grid_constant__ CUtensorMap tmap)
                              (int)((tile % p.ngroups) * G * 4), kb * 256, (int)(tile / p.ngroups));
         }
         bulk_commit();
+        grid_release();
         bulk_wait_read_all();
     }
 }

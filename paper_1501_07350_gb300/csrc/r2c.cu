@@ -146,7 +146,6 @@ __global__ void __launch_bounds__(kStageThreads) r2c_stage_kernel(const StageArg
     C* buf1 = buf0 + (size_t)n * ld;
     const int64_t L = p.M1, l0 = (int64_t)blockIdx.x * 2 * G;
     grid_wait();
-    grid_release();
     const T* x = reinterpret_cast<const T*>(p.in);
     {   // real lines l0 + 2j, l0 + 2j + 1 -> complex line j
         const int dj = kStageThreads / n, di = kStageThreads - dj * n;
@@ -190,7 +189,6 @@ __global__ void __launch_bounds__(kStageThreads) c2r_stage_kernel(const StageArg
     C* buf1 = buf0 + (size_t)n * ld;
     const int64_t L = p.M1, l0 = (int64_t)blockIdx.x * 2 * G;
     grid_wait();
-    grid_release();
     const typename RP::Scale ks = RP::scale_of(p.scale);
     {   // half lines l0 + 2j, l0 + 2j + 1 -> Hermitian-extended complex line j
         const int dj = kStageThreads / nh, dk = kStageThreads - dj * nh;
@@ -296,7 +294,6 @@ r2c_warp_kernel(const StageArgs p, int64_t ntiles)
     grid_wait();
     if (STAGED && t < ntiles) r2c_issue_raw<T, N>(x, L, t * TWO + 2 * warp, raw, lane);
     for (; t < ntiles; t += gridDim.x) {
-        if (t + gridDim.x >= ntiles) grid_release();
         const int64_t l0 = t * TWO;
         const int64_t la = l0 + 2 * warp, lb = la + 1;
         if constexpr (STAGED) {
@@ -390,7 +387,6 @@ c2r_warp_kernel(const StageArgs p, int64_t ntiles)
     grid_wait();
     if (staged && t < ntiles) c2r_issue_raw<A, NH>(in, L, t * 2 * G + 2 * warp, raw, lane);
     for (; t < ntiles; t += gridDim.x) {
-        if (t + gridDim.x >= ntiles) grid_release();
         const int64_t la = t * 2 * G + 2 * warp, lb = la + 1;
         if (staged) {
             cp_async_wait_all();

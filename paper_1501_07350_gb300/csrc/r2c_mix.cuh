@@ -175,7 +175,6 @@ real_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int64_t l0 = t * 2 * G, next = t + gridDim.x;
         const int nrow = rows(t);
-        if (next >= ntiles) grid_release();
         const bool mine = 2 * g < nrow, both = 2 * g + 1 < nrow;
         auto refill = [&]() { if (next < ntiles) copy_in(next); };
         cp_async_wait_all();
