@@ -109,7 +109,7 @@ batch_kernel(const BatchDev d, size_t buf_bytes)
         const int64_t t1 = t0 + d.tiles_per_item < ntile ? t0 + d.tiles_per_item : ntile;
         C* buf = reinterpret_cast<C*>(smem_raw);
         const int ld = Mix<A, G>::pitch(p.n);
-        mix_run<A, G, false>(p, s_plan, t0, 1, t1, buf, buf + G * ld, buf + 2 * G * ld, ld, kBatchThreads / G, kBatchThreads);
+        mix_run<A, G, false>(p, s_plan, t0, 1, t1, buf, buf + G * ld, buf + 2 * G * ld, ld, kBatchThreads / G, kBatchThreads, false);
         __threadfence();                           // release this thread's stores
         __syncthreads();
         if (tid == 0) atomicAdd(&d.done[q], 1u);

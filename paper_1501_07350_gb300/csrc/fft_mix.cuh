@@ -208,15 +208,19 @@ struct Mix {
 
 // Tiles tile, tile + step, ... below end of a stage, by a CTA of T threads.  cur and
 // oth: two tile buffers of G ld elements; tw: n elements for the length's twiddle
-// table, copied in here.  Returns with the CTA's threads still reading the buffers.
+// table, copied in here.  rows: the last pass, whose lines go out as they are, takes
+// consecutive threads along a line.  Returns with the CTA's threads still reading the
+// buffers.
 template <class A, int G, bool REPEAT>
 __device__ __forceinline__ void mix_run(const StageArgs& p, const MixPlan& plan, int64_t tile, int64_t step, int64_t end,
-                                        typename A::C* cur, typename A::C* oth, typename A::C* tw, int ld, int slots, int T)
+                                        typename A::C* cur, typename A::C* oth, typename A::C* tw, int ld, int slots, int T,
+                                        bool rows)
 {
     using M = Mix<A, G>;
     using C = typename A::C;
     const int tid = threadIdx.x;
     const int g = M::line_of(tid), slot = M::slot_of(tid), at = g * ld;
+    const int gl = rows ? tid / slots : g, sl = rows ? tid - gl * slots : slot, al = gl * ld;      // of the last pass
     TileGeom tg = tile_geom<REPEAT>(p, tile, G);
     for (int i = tid; i < p.n; i += T) cp_async<M::E>(tw + i, reinterpret_cast<const C*>(p.tw) + i);
     M::issue_load(p, tg.line0, tg.lstride, tg.valid, cur, ld, tid, T);
@@ -237,10 +241,10 @@ __device__ __forceinline__ void mix_run(const StageArgs& p, const MixPlan& plan,
             }
             // every thread has read `cur`: it takes the next tile while the last pass runs
             if (next < end) M::issue_load(p, tn.line0, tn.lstride, tn.valid, cur, ld, tid, T);
-            if (mine) M::template dispatch<false>(p, plan.pass[np - 1], true, tg, oth + at, cur + at, tw, g, slot, slots);
+            if (gl < tg.valid) M::template dispatch<false>(p, plan.pass[np - 1], true, tg, oth + al, cur + al, tw, gl, sl, slots);
         } else {
             if (next < end) M::issue_load(p, tn.line0, tn.lstride, tn.valid, oth, ld, tid, T);
-            if (mine) M::template dispatch<true>(p, plan.pass[0], true, tg, cur + at, oth + at, tw, g, slot, slots);
+            if (gl < tg.valid) M::template dispatch<true>(p, plan.pass[0], true, tg, cur + al, oth + al, tw, gl, sl, slots);
             C* t = cur; cur = oth; oth = t;
         }
         tg = tn;
@@ -250,7 +254,7 @@ __device__ __forceinline__ void mix_run(const StageArgs& p, const MixPlan& plan,
 
 template <class A, int G, bool REPEAT>
 __global__ void __launch_bounds__(kMixMaxThreads, mix_min_ctas())
-fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t ntiles)
+fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t ntiles, bool rows)
 {
     using C = typename A::C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -259,7 +263,7 @@ fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t 
     grid_wait();
     // the grid has at most ntiles CTAs
     mix_run<A, G, REPEAT>(p, plan, blockIdx.x, gridDim.x, ntiles, buf, buf + G * ld, buf + 2 * G * ld, ld, plan.slots,
-                          blockDim.x);
+                          blockDim.x, sizeof(C) == 8 && rows);
 }
 
 // The radix plan of length n for a policy of 16-byte (double-float) or 8-byte (FP32)

@@ -90,7 +90,15 @@ cudaError_t launch_mix_r(const StageLaunch& L, cudaStream_t st, bool* handled)
     if (ntiles > 0x7fffffffLL) return cudaSuccess;      // tiles are counted in 32 bits
     *handled = true;
     const int64_t grid = tile_grid<A>(ntiles, (int64_t)L.sms * ml.per_sm);
-    return launch_chained(kern, (unsigned)grid, ml.threads, ml.smem, st, a, ml.plan, ntiles);
+    // FP32 stages of contiguous output: with lines across the lanes a warp's store of the
+    // last pass touches 8 lines of 128 bytes, and the stage took 68 us of 256^3 (transposed
+    // ones 53), bound by its stores' wavefronts; along a line it touches two, for a few
+    // conflicts of its twiddle loads.  256^3 154.5 -> 138.5 us, 512^3 1450 -> 1311,
+    // 240x288x320 213 -> 192, 180x200x225 83.8 -> 80.6; where the pass has butterflies for
+    // fewer than 7 of 8 threads of a line it gains nothing.  A choice at run time: as a
+    // kernel of its own, whose code each transform loads anew, 256^3 took 149.5.
+    const bool rows = a.contig_store && ml.plan.pass[ml.plan.npass - 1].nbf * 8 >= ml.plan.slots * 7;
+    return launch_chained(kern, (unsigned)grid, ml.threads, ml.smem, st, a, ml.plan, ntiles, rows);
 }
 
 template <class A, int G>
