@@ -15,11 +15,14 @@ cudaError_t launch_tile_df(const StageLaunch& L, cudaStream_t st, bool* handled)
         cudaError_t e = L.args.n == 256 ? launch_warp_tma_256(L, st, handled) : launch_warp_tma_512(L, st, handled);
         if (*handled || e) return e;
     }
-    // a 32-point tile of the warp kernel is one warp: with few lines it leaves the
-    // chip nearly empty, and fft_mix's 128-thread tiles are faster (32^3 10.5 against
-    // 11.8 us, 64x32x32 11.9 against 14.4; 128x64x32, 8192 lines, the same; above, the
-    // warp kernel: 128x128x32 23 against 31)
-    if (L.family == KERNEL_AUTO && L.args.n == 32 && L.args.M1 * L.args.M2 <= 4096) {
+    // a tile of the warp kernel is one warp of 32-point lines, two of 64-point ones: with
+    // few lines it leaves the chip nearly empty, and fft_mix's tiles are faster (32^3 10.5
+    // against 11.8 us; with 64-point lines on it too, 64x32x32 10.9 against 12.8, 32x32x64
+    // 10.5 against 12.2, 64x64x32 11.8 against 13.3).  Above, the warp kernel: 64^3, 4096
+    // lines, 13.5 against 15.2, 32x32x256, 8192 of 32 points, 14.5 against 16.0, 128x128x32
+    // 21.5 against 25.4.
+    const int64_t lines = L.args.M1 * L.args.M2;
+    if (L.family == KERNEL_AUTO && ((L.args.n == 32 && lines <= 4096) || (L.args.n == 64 && lines <= 2048))) {
         cudaError_t e = launch_mix_df(L, st, handled);
         if (*handled || e) return e;
     }

@@ -11,10 +11,10 @@ cudaError_t launch_tile_f32(const StageLaunch& L, cudaStream_t st, bool* handled
     // fft_mix also beats the warp kernel on the longer power-of-two lengths (256^3 156
     // against 172-198 us, 512^3 1460 against 1590-1650) and on 64 and 128 points where
     // there are lines enough to fill the chip several times (512x64x512 183 against
-    // 194, 512x128x512 354 against 362); 64^3 (4096 lines) takes 10.7 against 8-9 us
-    // and 128^3 (16384) 28.2 against 26.3
+    // 194, 512x128x512 354 against 362; 128^3, 16384 lines, 24.0 against 25.7).  64^3 (4096
+    // lines) takes 10.0 against 7.4 us, 128x128x64 (8192 to 16384) 14.5 against 14.0.
     const int64_t lines = L.args.M1 * L.args.M2;
-    if (L.family == KERNEL_AUTO && (L.args.n >= 256 || (L.args.n >= 64 && lines >= 32768))) {
+    if (L.family == KERNEL_AUTO && (L.args.n >= 256 || (L.args.n == 64 && lines >= 32768) || (L.args.n == 128 && lines >= 16384))) {
         cudaError_t e = launch_mix_f32(L, st, handled);
         if (*handled || e) return e;
     }
