@@ -3,23 +3,30 @@
 // double-float and the FP32 arithmetic.
 //
 // A CTA takes tiles of G lines.  The radix plan is chosen on the host per length
-// (mix_plan): few passes of large radices (composite ones up to 10 in
+// (mix_radix_plan): few passes of large radices (composite ones up to 10 in
 // double-float, 16 in FP32, whose coprime factors need no twiddles between
 // them), each pass compiled per radix, strides and counts at run time.
 //
-// Tile layout in shared memory: [position][G lines], so the lanes of a warp take
-// consecutive lines at one position: every pass reads and writes rows of
-// G elements whatever the radix and the length, a twiddle is one broadcast load
-// for the G lines (from the CTA's own copy of the length's table), and the last pass's results leave for global memory straight
-// from registers, G consecutive elements per frequency (the transposed store) or
-// 32 / G consecutive frequencies per line (the contiguous one).  Rows of 128 bytes
-// are padded by one element, so that the copies in (lanes along a line) are free
-// of bank conflicts too; rows of 64 bytes are not, and their copies run with
-// lanes across the lines (two consecutive positions fill the banks).
+// Tile layout in shared memory: line after line, padded so that consecutive lines
+// start one or two elements apart in the banks, and the lanes of a warp take
+// consecutive lines at one position (two consecutive positions, where G lines do
+// not fill the banks): every pass reads and writes without conflicts whatever the
+// radix and the length, a twiddle is one broadcast load for the G lines (from the CTA's own
+// copy of the length's table), the copies in run along the lines, and the last pass's
+// results leave for global memory straight from registers, G consecutive elements per
+// frequency (the transposed store).  FP32 lines of contiguous output have their last
+// pass run along the line instead (fft_mix_launch.cuh).
 //
-// Passes alternate between two tile buffers, one barrier each.  The last pass reads
+// Passes alternate between two tile buffers, one barrier each (in place, with a barrier
+// between a pass's reads and writes, the radix cases spilled).  The last pass reads
 // one buffer and writes global memory, so the next tile's copies (cp.async) go into
 // the other buffer while it runs.
+//
+// In double-float the instructions bound it (6.5-8.5 a point and stage, 47-55 % of issue
+// slots) with the barriers between passes; FP32 runs at 75-85 % of the copy bandwidth on
+// large arrays.  Against the kernels before it (compile-time mixed radices, generic), us:
+// 240x288x320 complex128 1317 -> 774, complex64 452 -> 193; 120x144x160 complex128 137 ->
+// 99; 180x200x225 complex64 183 -> 81; 98x343x105 complex128 330 -> 172.
 #pragma once
 #include <type_traits>
 
