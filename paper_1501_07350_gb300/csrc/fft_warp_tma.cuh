@@ -289,7 +289,7 @@ fft_warp_tma_kernel(const StageArgs p, const __grid_constant__ CUtensorMap tmap)
         }
         bulk_commit();
         grid_release();
-        bulk_wait_read_all();
+        bulk_wait_read_all();          // the shared memory is free; the grid's end completes the writes
     }
 }
 
