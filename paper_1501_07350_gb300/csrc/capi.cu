@@ -922,6 +922,7 @@ StageLaunch stage_lines(const StageLaunch& L, int64_t u0, int64_t u1, int64_t* i
     StageLaunch c = L;
     StageArgs& a = c.args;
     const int64_t whole = a.M1 * a.M2 * (int64_t)a.n;
+    c.stage_lines = choice_lines(L);
     if (a.M2 > 1) {
         *in_off = u0 * a.M1 * a.n; *out_off = u0 * a.S2; *lines = (u1 - u0) * a.M1;
         a.M2 = u1 - u0;

@@ -65,7 +65,14 @@ struct StageLaunch {
     int sms;                   // multiprocessors of the device (persistent grids)
     int family;                // KERNEL_*: which stage kernel runs this launch
     int* status;               // device status word (DFT-GEMM stages)
+    // lines of the stage that this launch is a range of (0: it is the whole stage)
+    int64_t stage_lines = 0;
 };
+
+// Lines that the choice of a stage's kernel goes by.  A range of lines takes the kernel
+// of its whole stage: the kernels round differently, and openfft_exec_c2c_host, which
+// runs the first and the last stage range by range, gives openfft_exec_c2c's bits.
+inline int64_t choice_lines(const StageLaunch& L) { return L.stage_lines ? L.stage_lines : L.args.M1 * L.args.M2; }
 
 // stage kernel families: warp-per-line (power-of-two n), tile (specialised n),
 // generic (any n); AUTO takes the first that has an instantiation for (n, G)

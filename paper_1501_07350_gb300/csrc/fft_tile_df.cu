@@ -21,7 +21,7 @@ cudaError_t launch_tile_df(const StageLaunch& L, cudaStream_t st, bool* handled)
     // 10.5 against 12.2, 64x64x32 11.8 against 13.3).  Above, the warp kernel: 64^3, 4096
     // lines, 13.5 against 15.2, 32x32x256, 8192 of 32 points, 14.5 against 16.0, 128x128x32
     // 21.5 against 25.4.
-    const int64_t lines = L.args.M1 * L.args.M2;
+    const int64_t lines = choice_lines(L);
     if (L.family == KERNEL_AUTO && ((L.args.n == 32 && lines <= 4096) || (L.args.n == 64 && lines <= 2048))) {
         cudaError_t e = launch_mix_df(L, st, handled);
         if (*handled || e) return e;

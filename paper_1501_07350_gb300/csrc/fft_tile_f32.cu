@@ -13,7 +13,7 @@ cudaError_t launch_tile_f32(const StageLaunch& L, cudaStream_t st, bool* handled
     // there are lines enough to fill the chip several times (512x64x512 183 against
     // 194, 512x128x512 354 against 362; 128^3, 16384 lines, 24.0 against 25.7).  64^3 (4096
     // lines) takes 10.0 against 7.4 us, 128x128x64 (8192 to 16384) 14.5 against 14.0.
-    const int64_t lines = L.args.M1 * L.args.M2;
+    const int64_t lines = choice_lines(L);
     if (L.family == KERNEL_AUTO && (L.args.n >= 256 || (L.args.n == 64 && lines >= 32768) || (L.args.n == 128 && lines >= 16384))) {
         cudaError_t e = launch_mix_f32(L, st, handled);
         if (*handled || e) return e;

@@ -199,3 +199,27 @@ def test_copy_streams_errors_and_reset(torch):
             assert np.array_equal(_bits(y), _bits(want))
     finally:
         of.openfft_destroy(plan)
+
+
+# Stages on either side of the line counts at which the choice of a stage's kernel
+# changes (32 points at 4096 lines and 64 at 2048 in double-float; 64 at 32768 and 128
+# at 16384 in FP32): their ranges have fewer lines than the stage, which decides.
+@pytest.mark.parametrize("shape,dtype", [((32, 128, 32), of.C2C_F64), ((32, 160, 32), of.C2C_F64), ((64, 32, 64), of.C2C_F64),
+                                         ((64, 64, 64), of.C2C_F64), ((64, 512, 64), of.C2C_F32), ((64, 500, 64), of.C2C_F32),
+                                         ((128, 128, 128), of.C2C_F32), ((128, 120, 128), of.C2C_F32)])
+def test_ranges_take_the_kernel_of_their_stage(torch, shape, dtype):
+    x = synth.complex_field(shape, seed=shape[1]).reshape(-1)
+    x = x if dtype == of.C2C_F64 else x.astype(np.complex64)
+    hx = torch.from_numpy(x).pin_memory()
+    hy = torch.empty_like(hx).pin_memory()
+    plan = of.openfft_plan(*shape, 1, dtype)
+    try:
+        for direction in (of.FORWARD, of.BACKWARD):
+            want = _device(torch, plan, x, direction)
+            for chunks in (0, 1, 5, 32):
+                of.openfft_set_host_chunks(plan, chunks)
+                hy.fill_(float("nan"))
+                of.openfft_exec_c2c_host(plan, hx.numpy(), hy.numpy(), direction)
+                assert np.array_equal(_bits(hy.numpy()), _bits(want)), (chunks, direction)
+    finally:
+        of.openfft_destroy(plan)
