@@ -13,6 +13,10 @@ namespace ofg {
 
 // ------------------------------------------------ element load / store ----
 
+// load() reads data that an earlier stage of the chain wrote.  That stage may still have
+// been running when this kernel's CTAs became resident (grid_wait, fft_stage.h), so these
+// are plain loads: the read-only path (__ldg) wants data that nothing writes during the
+// kernel, and grid_wait does not order it.
 template <class A> struct Io;
 
 template <> struct Io<ArF64> {
@@ -22,7 +26,7 @@ template <> struct Io<ArF64> {
     __device__ __forceinline__ static void store_mid(void* p, double2 v) { *reinterpret_cast<double2*>(p) = v; }
     __device__ __forceinline__ static double2 from_c128(double2 v) { return v; }
     __device__ __forceinline__ static double2 load(const void* p, int, int64_t i) {
-        return __ldg(reinterpret_cast<const double2*>(p) + i);
+        return reinterpret_cast<const double2*>(p)[i];
     }
     __device__ __forceinline__ static void store(void* p, int, int64_t i, double2 v) {
         reinterpret_cast<double2*>(p)[i] = v;
@@ -36,7 +40,7 @@ template <> struct Io<ArF32> {
     __device__ __forceinline__ static void store_mid(void* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
     __device__ __forceinline__ static float2 from_c128(double2 v) { return make_float2((float)v.x, (float)v.y); }
     __device__ __forceinline__ static float2 load(const void* p, int, int64_t i) {
-        return __ldg(reinterpret_cast<const float2*>(p) + i);
+        return reinterpret_cast<const float2*>(p)[i];
     }
     __device__ __forceinline__ static void store(void* p, int, int64_t i, float2 v) {
         reinterpret_cast<float2*>(p)[i] = v;
@@ -127,8 +131,8 @@ template <> struct Io<ArDF> {
     __device__ __forceinline__ static void store_mid(void* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
     __device__ __forceinline__ static float4 from_c128(double2 v) { return df_from_double2(v); }
     __device__ __forceinline__ static float4 load(const void* p, int fmt, int64_t i) {
-        if (fmt == FMT_DF) return __ldg(reinterpret_cast<const float4*>(p) + i);
-        return df_from_double2(__ldg(reinterpret_cast<const double2*>(p) + i));
+        if (fmt == FMT_DF) return reinterpret_cast<const float4*>(p)[i];
+        return df_from_double2(reinterpret_cast<const double2*>(p)[i]);
     }
     __device__ __forceinline__ static void store(void* p, int fmt, int64_t i, float4 v) {
         if (fmt == FMT_DF) reinterpret_cast<float4*>(p)[i] = v;

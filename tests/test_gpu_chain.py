@@ -98,3 +98,81 @@ def test_a_cta_per_tile(torch, n, other):
                 assert err < 1e-12, (shape, direction, err)
         finally:
             plan.close()
+
+
+# Chains whose stale data is wrong data: two inputs in turn, every buffer filled with NaN
+# before its first run, results copied in stream order; then replays of a captured chain
+# whose input changes between them, beside work on a second stream.  Real plans run each
+# of their last stages: the warp kernels (512 points in float load without staging), the
+# generic stage (under 2^15 points) and the any-length kernel.
+@pytest.mark.parametrize("shape,dtype", [(s, d) for s in SHAPES for d in (of.C2C_F64, of.C2C_F32)] +
+                         [(s, d) for s in ((8, 4, 512), (16, 64, 128), (9, 10, 15), (40, 36, 30), (24, 20, 256))
+                          for d in (of.R2C_F64, of.R2C_F32)])
+def test_chains_on_changing_inputs(torch, shape, dtype):
+    real = dtype in (of.R2C_F64, of.R2C_F32)
+    wide = dtype in (of.C2C_F64, of.R2C_F64)
+    ct = torch.complex128 if wide else torch.complex64
+    n, half = int(np.prod(shape)), shape[0] * shape[1] * (shape[2] // 2 + 1)
+    xt = (torch.float64 if wide else torch.float32) if real else ct
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    xs = [torch.randn(n, generator=gen, device="cuda", dtype=xt) for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    plans = [of.Plan(*shape, 2, dtype, stream=s) for s in streams]
+
+    def buffers():
+        sizes = [(half, ct), (n, xt), (half, ct)] if real else [(n, ct)] * 3
+        return [torch.full((m,), float("nan"), device="cuda", dtype=t) for m, t in sizes]
+
+    def steps(plan, x, b):
+        if real:
+            return [lambda: of.openfft_exec_r2c(plan.handle, x, b[0]), lambda: of.openfft_exec_c2r(plan.handle, b[0], b[1]),
+                    lambda: of.openfft_exec_r2c(plan.handle, b[1], b[2])]
+        return [lambda: plan.exec(x, b[0], of.FORWARD), lambda: plan.exec(b[0], b[1], of.BACKWARD),
+                lambda: plan.exec(b[1], b[2], of.FORWARD)]
+
+    def equal(got, want):
+        parts = lambda t: torch.view_as_real(t) if t.is_complex() else t
+        return all(torch.equal(parts(g), parts(w)) for g, w in zip(got, want))
+
+    want = []
+    for x in xs:
+        b = buffers()
+        torch.cuda.synchronize()
+        for step in steps(plans[0], x, b):
+            step()
+            torch.cuda.synchronize()
+        want.append(b)
+    bufs = [buffers() for _ in plans]
+    torch.cuda.synchronize()
+    got = [[], []]
+    for k in range(6):
+        for i, p in enumerate(plans):
+            for step in steps(p, xs[(k + i) % 2], bufs[i]):
+                step()
+            with torch.cuda.stream(streams[i]):
+                got[i].append([b.clone() for b in bufs[i]])
+    torch.cuda.synchronize()
+    for i in range(2):
+        for k in range(6):
+            assert equal(got[i][k], want[(k + i) % 2]), (i, k)
+    x, b = xs[0].clone(), buffers()
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=streams[0]):
+        for step in steps(plans[0], x, b):
+            step()
+    got, beside = [], []
+    for k in range(4):
+        with torch.cuda.stream(streams[0]):
+            x.copy_(xs[k % 2])
+            graph.replay()
+            got.append([t.clone() for t in b])
+        for step in steps(plans[1], xs[1 - k % 2], bufs[1]):
+            step()
+        with torch.cuda.stream(streams[1]):
+            beside.append([t.clone() for t in bufs[1]])
+    torch.cuda.synchronize()
+    for k in range(4):
+        assert equal(got[k], want[k % 2]) and equal(beside[k], want[1 - k % 2]), k
+    for p in plans:
+        p.close()
