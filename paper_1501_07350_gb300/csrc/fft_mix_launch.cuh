@@ -98,7 +98,7 @@ cudaError_t launch_mix_r(const StageLaunch& L, cudaStream_t st, bool* handled)
     // fewer than 7 of 8 threads of a line it gains nothing.  A choice at run time: as a
     // kernel of its own, whose code each transform loads anew, 256^3 took 149.5.
     const bool rows = a.contig_store && ml.plan.pass[ml.plan.npass - 1].nbf * 8 >= ml.plan.slots * 7;
-    return launch_chained(kern, (unsigned)grid, ml.threads, ml.smem, st, a, ml.plan, ntiles, rows);
+    return launch_chained(L, kern, (unsigned)grid, ml.threads, ml.smem, st, a, ml.plan, ntiles, rows);
 }
 
 template <class A, int G>

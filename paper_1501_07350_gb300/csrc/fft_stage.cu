@@ -196,9 +196,9 @@ cudaError_t launch_stage(const StageLaunch& L0, cudaStream_t st)
     }
     const unsigned grid = (unsigned)L.grid;
     switch (L.arith) {
-    case ARITH_F64: return launch_chained(fft_stage_kernel<ArF64>, grid, kStageThreads, L.smem, st, L.args);
-    case ARITH_F32: return launch_chained(fft_stage_kernel<ArF32>, grid, kStageThreads, L.smem, st, L.args);
-    default: return launch_chained(fft_stage_kernel<ArDF>, grid, kStageThreads, L.smem, st, L.args);
+    case ARITH_F64: return launch_chained(L, fft_stage_kernel<ArF64>, grid, kStageThreads, L.smem, st, L.args);
+    case ARITH_F32: return launch_chained(L, fft_stage_kernel<ArF32>, grid, kStageThreads, L.smem, st, L.args);
+    default: return launch_chained(L, fft_stage_kernel<ArDF>, grid, kStageThreads, L.smem, st, L.args);
     }
 }
 

@@ -67,6 +67,10 @@ struct StageLaunch {
     int* status;               // device status word (DFT-GEMM stages)
     // lines of the stage that this launch is a range of (0: it is the whole stage)
     int64_t stage_lines = 0;
+    // 1: the launch waits until the kernel before it has ended.  For a stage whose twiddle
+    // table that kernel writes: the stage kernels read tables through the read-only path,
+    // which wants them complete before the kernel is resident.
+    int apart = 0;
 };
 
 // Lines that the choice of a stage's kernel goes by.  A range of lines takes the kernel
@@ -101,11 +105,12 @@ cudaError_t launch_real_mix(const StageLaunch& L, cudaStream_t st, bool* handled
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... Args>
-cudaError_t launch_chained(void (*kern)(P...), unsigned grid, int threads, size_t smem, cudaStream_t st, const Args&... args)
+cudaError_t launch_chained(const StageLaunch& L, void (*kern)(P...), unsigned grid, int threads, size_t smem, cudaStream_t st,
+                           const Args&... args)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+    attr.val.programmaticStreamSerializationAllowed = L.apart ? 0 : 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3((unsigned)threads);

@@ -359,7 +359,7 @@ cudaError_t launch_tile_n(const StageLaunch& L, cudaStream_t st)
     int64_t grid = (int64_t)L.sms * blocks_per_sm;
     if (grid > ntiles) grid = ntiles;
     if (grid < 1) grid = 1;
-    return launch_chained(fft_tile_kernel<A, N, G, T>, (unsigned)grid, T, smem, st, L.args, ntiles);
+    return launch_chained(L, fft_tile_kernel<A, N, G, T>, (unsigned)grid, T, smem, st, L.args, ntiles);
 }
 
 // Launch the specialised kernel for (N, G) if there is one; *handled = false otherwise.

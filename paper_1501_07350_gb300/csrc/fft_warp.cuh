@@ -310,7 +310,7 @@ cudaError_t launch_warp_n(const StageLaunch& L, cudaStream_t st)
     }
     const int64_t ntiles = L.grid;
     const int64_t grid = tile_grid<A>(ntiles, (int64_t)L.sms * blocks_per_sm);
-    return launch_chained(fft_warp_kernel<A, N, G>, (unsigned)grid, T, smem, st, L.args, ntiles);
+    return launch_chained(L, fft_warp_kernel<A, N, G>, (unsigned)grid, T, smem, st, L.args, ntiles);
 }
 
 // power-of-two lengths go to the warp-per-line kernel

@@ -353,7 +353,7 @@ cudaError_t launch_warp_tma_v(const StageLaunch& L, const CUtensorMap& map, cuda
         if (e) return e;
         if (slot) *slot = 1;
     }
-    return launch_chained(kern, (unsigned)L.grid, 32 * G * tma_wpl<N>(), smem, st, L.args, map);
+    return launch_chained(L, kern, (unsigned)L.grid, 32 * G * tma_wpl<N>(), smem, st, L.args, map);
 }
 
 // The asynchronous-output kernel for n = 256 / 512 in tiles of G lines,

@@ -182,6 +182,7 @@ extern "C" int openfft_exec_c2c_noalloc(int Na, int Nb, int Nc, int P, int dtype
     L[0].args.in = in;      L[0].args.out = scratch;
     L[1].args.in = scratch; L[1].args.out = out;
     L[2].args.in = out;     L[2].args.out = out;
+    L[0].apart = 1;                            // after the twiddle kernels; stages 2 and 3 follow it
     for (int i = 0; i < 3; ++i)
         if ((e = launch_stage(L[i], s))) return cuda_fail(e);
     return OPENFFT_OK;

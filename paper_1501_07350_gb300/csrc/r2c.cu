@@ -447,8 +447,8 @@ cudaError_t launch_real_warp(const StageLaunch& L, cudaStream_t st)
     }
     const int64_t ntiles = (L.args.M1 + 2 * G - 1) / (2 * G);
     const int64_t grid = tile_grid<A>(ntiles, (int64_t)L.sms * per_sm);
-    return fwd ? launch_chained(r2c_warp_kernel<A, N, G>, (unsigned)grid, 32 * G, smem, st, L.args, ntiles)
-               : launch_chained(c2r_warp_kernel<A, N, G>, (unsigned)grid, 32 * G, smem, st, L.args, ntiles);
+    return fwd ? launch_chained(L, r2c_warp_kernel<A, N, G>, (unsigned)grid, 32 * G, smem, st, L.args, ntiles)
+               : launch_chained(L, c2r_warp_kernel<A, N, G>, (unsigned)grid, 32 * G, smem, st, L.args, ntiles);
 }
 
 // AW: the policy of the warp kernels
@@ -473,7 +473,7 @@ cudaError_t launch_real_a(const StageLaunch& L, cudaStream_t st)
             if (e) return e;
             if (slot) *slot = 1;
         }
-        return launch_chained(r2c_stage_kernel<A>, grid, kStageThreads, L.smem, st, L.args);
+        return launch_chained(L, r2c_stage_kernel<A>, grid, kStageThreads, L.smem, st, L.args);
     } else {
         int* slot = device_slot(attr_c2r);
         if (!slot || !*slot) {
@@ -482,7 +482,7 @@ cudaError_t launch_real_a(const StageLaunch& L, cudaStream_t st)
             if (e) return e;
             if (slot) *slot = 1;
         }
-        return launch_chained(c2r_stage_kernel<A>, grid, kStageThreads, L.smem, st, L.args);
+        return launch_chained(L, c2r_stage_kernel<A>, grid, kStageThreads, L.smem, st, L.args);
     }
 }
 

@@ -32,8 +32,8 @@ cudaError_t launch_real_g(const StageLaunch& L, cudaStream_t st, bool* handled)
     const int64_t ntiles = (L.args.M1 + 2 * G - 1) / (2 * G);
     // 180x200x225 double forward 200 us with one share a CTA, 195 with 4, 201 with 8
     const unsigned grid = (unsigned)tile_grid<A>(ntiles, (int64_t)L.sms * ml.per_sm, 4);
-    return fwd ? launch_chained(real_mix_kernel<A, G, true>, grid, ml.threads, ml.smem, st, L.args, ml.plan, ntiles)
-               : launch_chained(real_mix_kernel<A, G, false>, grid, ml.threads, ml.smem, st, L.args, ml.plan, ntiles);
+    return fwd ? launch_chained(L, real_mix_kernel<A, G, true>, grid, ml.threads, ml.smem, st, L.args, ml.plan, ntiles)
+               : launch_chained(L, real_mix_kernel<A, G, false>, grid, ml.threads, ml.smem, st, L.args, ml.plan, ntiles);
 }
 
 }  // namespace

@@ -176,3 +176,31 @@ def test_chains_on_changing_inputs(torch, shape, dtype):
         assert equal(got[k], want[k % 2]) and equal(beside[k], want[1 - k % 2]), k
     for p in plans:
         p.close()
+
+
+# The allocation-free call writes its twiddle tables ahead of its stages on every call, at
+# one place for all lengths: calls of different lengths back to back, on lengths whose
+# kernels read the tables where they are (warp kernels) and whose kernels copy them.
+@pytest.mark.parametrize("dtype", [of.C2C_F64, of.C2C_F32])
+def test_noalloc_calls_of_different_lengths_back_to_back(torch, dtype):
+    tdt = torch.complex128 if dtype == of.C2C_F64 else torch.complex64
+    shapes = [(64, 64, 64), (128, 64, 32), (32, 256, 64), (64, 48, 100), (128, 32, 128), (36, 40, 30)]
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    xs = [torch.randn(int(np.prod(s)), generator=gen, device="cuda", dtype=tdt) for s in shapes]
+    stream = torch.cuda.current_stream()
+
+    def run(shape, x, direction):
+        y = torch.full_like(x, float("nan"))
+        of.openfft_exec_c2c_noalloc(*shape, 1, dtype, x, y, direction, stream)
+        return y
+
+    calls = [(s, x, d) for s, x in zip(shapes, xs) for d in (of.FORWARD, of.BACKWARD)]
+    want = []
+    for c in calls:
+        torch.cuda.synchronize()
+        want.append(run(*c))
+    torch.cuda.synchronize()
+    got = [run(*c) for _ in range(3) for c in calls]
+    torch.cuda.synchronize()
+    for k, g in enumerate(got):
+        assert torch.equal(torch.view_as_real(g), torch.view_as_real(want[k % len(calls)])), calls[k % len(calls)][0]
