@@ -35,6 +35,7 @@
 #include "batch.h"
 #include "fft_stage.h"
 #include "batch_kernel.cuh"
+#include "fft_mix_launch.cuh"
 
 namespace ofg {
 
@@ -194,8 +195,11 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
     }
     // launch shape: persistent, as many CTAs as fit (tile buffer + queue tables)
     if (b->smem + tables > 200 * 1024) { free_batch(b); return fail(OPENFFT_ERR_UNSUPPORTED, "batch too large for the queue tables in shared memory"); }
+    // The kernel's shared-memory limit is the same for every plan: plans of other sizes share
+    // the kernel, and this one's launches are captured at its first calls.
     int per_sm = 1;
-    e = persistent_ctas_per_sm(kernel_of(f32, b->G), kBatchThreads, b->smem + tables, &per_sm);
+    e = prepare_kernel(kernel_of(f32, b->G), nullptr);
+    if (!e) e = resident_ctas_per_sm(kernel_of(f32, b->G), kBatchThreads, b->smem + tables, &per_sm);
     if (e) { free_batch(b); return fail(OPENFFT_ERR_CUDA, cudaGetErrorString(e)); }
     b->grid = sms * (per_sm > 0 ? per_sm : 1);
     {

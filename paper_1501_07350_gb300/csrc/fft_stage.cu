@@ -93,16 +93,12 @@ __global__ void warp_twiddle_kernel(int n, void* out)
 
 // --------------------------------------------------------- host side ----
 
-cudaError_t persistent_ctas_per_sm(const void* func, int threads, size_t dyn_smem, int* per_sm)
+cudaError_t resident_ctas_per_sm(const void* func, int threads, size_t dyn_smem, int* per_sm, int* carveout)
 {
     // cudaOccupancyMaxActiveBlocksPerMultiprocessor has been seen to count one
-    // CTA per SM where two were resident, so the limits are applied here; the
-    // carveout is then set to what those CTAs need, leaving the rest as L1
-    // (which the twiddle loads use)
-    cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_smem);
+    // CTA per SM where two were resident, so the limits are applied here
     cudaFuncAttributes fa;
-    if (!e) e = cudaFuncGetAttributes(&fa, func);
-    if (e) return e;
+    if (cudaError_t e = cudaFuncGetAttributes(&fa, func)) return e;
     int dev = 0, smem_sm = 0, resv = 0, regs_sm = 0, thr_sm = 0, blk_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
@@ -119,10 +115,18 @@ cudaError_t persistent_ctas_per_sm(const void* func, int threads, size_t dyn_sme
     n = std::min(n, (long)thr_sm / (32 * warps));
     if (n < 1) n = 1;
     *per_sm = (int)n;
-    if (smem_sm > 0) {
-        const long pct = std::min(100L, (100 * n * cta_smem + smem_sm - 1) / smem_sm + 2);
-        e = cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, (int)pct);
-    }
+    if (carveout) *carveout = smem_sm > 0 ? (int)std::min(100L, (100 * n * cta_smem + smem_sm - 1) / smem_sm + 2) : -1;
+    return cudaSuccess;
+}
+
+cudaError_t persistent_ctas_per_sm(const void* func, int threads, size_t dyn_smem, int* per_sm)
+{
+    // the carveout is set to what the CTAs need, leaving the rest as L1 (which the
+    // twiddle loads use)
+    int pct = -1;
+    cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_smem);
+    if (!e) e = resident_ctas_per_sm(func, threads, dyn_smem, per_sm, &pct);
+    if (!e && pct >= 0) e = cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
     return e;
 }
 

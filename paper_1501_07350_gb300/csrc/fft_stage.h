@@ -130,7 +130,10 @@ cudaError_t dev_malloc(void** ptr, size_t bytes);
 // Resident CTAs per SM of a persistent kernel with `threads` threads and
 // `dyn_smem` bytes of dynamic shared memory, from the kernel's own limits
 // (shared memory with the whole carveout as shared memory, registers,
-// threads); sets the kernel's dynamic shared memory limit and carveout.
+// threads); *carveout (if given) is the percentage that these CTAs need.
+cudaError_t resident_ctas_per_sm(const void* func, int threads, size_t dyn_smem, int* per_sm, int* carveout = nullptr);
+// The same for a kernel that is always launched with `dyn_smem` bytes; sets the kernel's
+// dynamic shared memory limit and carveout.
 cudaError_t persistent_ctas_per_sm(const void* func, int threads, size_t dyn_smem, int* per_sm);
 // Launch properties are cached per device (kernel attributes are per device):
 // the current device's slot of `slots`, or nullptr beyond kMaxDevices (then

@@ -134,3 +134,19 @@ def test_batch_tile_widths(torch, shapes, dtype, tol):
         _check_batch(torch, plan, shapes, Ps, xs, xd, dtype, tol)
     finally:
         of.openfft_destroy(plan)
+
+
+@pytest.mark.parametrize("dtype,tol", [(of.C2C_F32, 1e-5), (of.C2C_F64, 1e-12)])
+def test_plans_of_several_sizes_at_once(torch, dtype, tol):
+    """Plans that share a kernel and differ in shared memory, each first run in a
+    direction after a smaller or a larger one has been made."""
+    Ps = [1]
+    batches = [[(100, 108, 120)], [(16, 20, 24)], [(60, 50, 40)], [(2048, 3, 4)], [(1536, 2, 3)]]
+    plans = [of.openfft_plan_many(shapes, Ps, dtype) for shapes in batches]
+    try:
+        for plan, shapes in zip(plans, batches):
+            xs, xd = _inputs(torch, shapes, 31, dtype)
+            _check_batch(torch, plan, shapes, Ps, xs, xd, dtype, tol)
+    finally:
+        for plan in plans:
+            of.openfft_destroy(plan)
