@@ -21,13 +21,27 @@
 // and stores of different items in flight.  64 uneven complex64 transforms (48^3 to
 // 100x108x120) take 461 us, 797 with 256-thread CTAs and the specialised tile bodies
 // (272 would be three reads and writes at the measured copy rate); the same in
-// double-float 1534, 3253 before.  A CTA claims its next
+// double-float 1534, 3253 before.
+//
+// A batch with a long axis (over 564 points in FP32, 282 in double-float), or with so many
+// transforms that the queue tables fill the shared memory, holds one or two such CTAs on
+// an SM.  It runs on one CTA of 512 threads instead, where each stage has its own tile
+// width and the CTA's threads split into groups with a tile each, so that the short
+// axes beside a long one keep wide tiles and all of the threads.  One 2048x48x48 beside 63 48^3:
+// complex64 321 us (with 128-thread CTAs and one width for all stages 1282; generic body of
+// 256 threads, which it replaced, 705), complex128 567 (4279, 1882); 40 60^3 beside four
+// 1200x200x40 851 and 2393 (1904 and 7491); 4000 8^3 2099 and 2143 (2323 and 4273).  With
+// 64 registers and two CTAs an SM instead of 128 and one, complex128 took 1.2 to 2.1
+// times as long (spills), with 256 threads and three CTAs 1.1 to 2.5 times.
+//
+// A CTA claims its next
 // item before it starts on the current one, so the queue's atomic and the search are
 // not waited for.  A claimed item may stay behind one that waits for earlier items;
 // waits still end: the unfinished item with the lowest index is never behind another,
 // and everything it waits for has lower indices.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
@@ -45,20 +59,40 @@ namespace ofg {
 // with 16 tiles an item), 64 uneven ones 461 (472 with four items per CTA, 495 six).
 constexpr int kMaxTilesPerItem = 16;
 constexpr int kItemsPerCta = 2;
+// Shared memory of a CTA at most: tile buffers and queue tables.
+constexpr size_t kMaxBatchSmem = 201 * 1024;
 
 // --------------------------------------------------------------- host ----
 
+namespace {
+
 size_t tile_bytes_of(bool f32, int G, int n) { return f32 ? batch_tile_bytes_f32(G, n) : batch_tile_bytes_df(G, n); }
-const void* kernel_of(bool f32, int G) { return f32 ? batch_kernel_f32(G) : batch_kernel_df(G); }
+const void* kernel_of(bool f32, bool wide) { return f32 ? batch_kernel_f32(wide) : batch_kernel_df(wide); }
+int threads_of(bool wide) { return wide ? kBatchWideThreads : kBatchThreads; }
+
+// Tile width of a stage of lines of n points, Mg of them side by side in the output: at
+// most 8 lines, no more than there are, and what `budget` bytes of shared memory hold.
+int tile_width(bool f32, int n, int64_t Mg, size_t budget)
+{
+    int G = 8;
+    while (G > 1 && (G / 2 >= Mg || tile_bytes_of(f32, G, n) > budget)) G /= 2;
+    return G;
+}
+
+int64_t grouped_lines(const StageArgs& a) { return a.group_i2 ? a.M2 : a.M1; }
+int64_t tiles_of(const StageArgs& a) { return a.ngroups * (a.group_i2 ? a.M1 : a.M2); }
+
+}  // namespace
 
 struct BatchPlan {
-    int count = 0, dtype = 0, arith = 0, G = 8, tiles_per_item = 1;
+    int count = 0, dtype = 0, arith = 0;
+    bool wide = false;                         // the kernel of 512-thread CTAs
     std::vector<int> dims;                     // 3 * count
     std::vector<int64_t> N;                    // per transform
     size_t smem = 0;
     int grid = 0;
     // device memory
-    StageArgs* d_stages = nullptr;             // and the radix plans after them
+    BatchStage* d_stages = nullptr;            // and the radix plans after them
     int64_t* d_item_base = nullptr;
     unsigned* d_need = nullptr;
     void** d_ptrs = nullptr;
@@ -110,7 +144,7 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
     const int ext = dtype == OPENFFT_C2C_F32 ? FMT_C64 : FMT_C128;
     const int mid = dtype == OPENFFT_C2C_F32 ? FMT_C64 : FMT_DF;
     const int twf = dtype == OPENFFT_C2C_F32 ? FMT_C64 : FMT_DF;
-    std::vector<StageArgs> st((size_t)2 * 3 * count);
+    std::vector<BatchStage> st((size_t)2 * 3 * count);
     cudaError_t e;
     const bool f32 = dtype == OPENFFT_C2C_F32;
     // twiddle table and radix plan per distinct length
@@ -133,15 +167,6 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
         a.aux = reinterpret_cast<const void*>(k);        // its plan's index until the table has an address
         return OPENFFT_OK;
     };
-    // Lines per tile: 8 while an SM holds three CTAs of such tiles of the longest axis,
-    // else the fewest (4 in FP32, 2 in double-float, which fit every length).
-    const size_t tables = sizeof(int64_t) * (size_t)(3 * count + 1) + sizeof(unsigned) * (size_t)(3 * count);
-    int nmax = 1;
-    for (int i = 0; i < 3 * count; ++i) nmax = dims[i] > nmax && dims[i] <= kMaxLen ? dims[i] : nmax;
-    b->G = f32 ? 4 : 2;
-    for (int G : {8, 4})
-        if (((tile_bytes_of(f32, G, nmax) + 15) & ~(size_t)15) + tables <= 75 * 1024) { b->G = G; break; }
-    b->smem = (tile_bytes_of(f32, b->G, nmax) + 15) & ~(size_t)15;
     for (int i = 0; i < count; ++i) {
         const int64_t Na = dims[3 * i], Nb = dims[3 * i + 1], Nc = dims[3 * i + 2];
         if (Na < 1 || Nb < 1 || Nc < 1 || P[i] < 1) { free_batch(b); return fail(OPENFFT_ERR_INVALID_ARG, "sizes and P must be >= 1"); }
@@ -164,24 +189,42 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
         for (int dir = 0; dir < 2; ++dir)
             for (int s = 0; s < 3; ++s) {
                 const Geo& g = geo[dir][s];
-                StageArgs& a = st[(size_t)dir * 3 * count + (size_t)s * count + i];
-                std::memset(&a, 0, sizeof(a));
+                BatchStage& bs = st[(size_t)dir * 3 * count + (size_t)s * count + i];
+                std::memset(&bs, 0, sizeof(bs));
+                StageArgs& a = bs.args;
                 const int n = (int)g.n;
-                const int64_t Mg = g.g2 ? g.M2 : g.M1;
-                const int G = b->G;
                 if (const int status = tables_for(n, a)) { free_batch(b); return status; }
                 a.M1 = g.M1; a.M2 = g.M2; a.S1 = g.S1; a.S2 = g.S2; a.Sk = g.Sk;
-                a.ngroups = (Mg + G - 1) / G;
                 a.scale = g.scale;
                 split_scale(a);
-                a.n = n; a.G = G;
+                a.n = n;
                 a.group_i2 = g.g2; a.contig_store = g.contig;
                 a.conj_in = g.cin; a.conj_out = g.cout; a.do_fft = 1;
                 a.in_fmt = g.in_fmt; a.out_fmt = g.out_fmt;
             }
     }
+    // Kernel and tile widths.  CTAs of 128 threads and tiles of 8 lines for every stage, while
+    // an SM holds three CTAs with such tiles of the longest axis (and the queue tables).
+    // Otherwise one CTA of 512 threads an SM, whose shared memory every stage has to
+    // itself: the width is the most that fits, and the threads split into groups with a
+    // tile each, as many as fit beside each other.
+    const size_t tables = sizeof(int64_t) * (size_t)(3 * count + 1) + sizeof(unsigned) * (size_t)(3 * count);
+    int nmax = 1;
+    for (int v : b->dims) nmax = std::max(nmax, v);
+    b->wide = tile_bytes_of(f32, 8, nmax) + tables > 75 * 1024;
+    const size_t budget = tables < kMaxBatchSmem ? kMaxBatchSmem - tables : 0;
+    for (BatchStage& bs : st) {
+        StageArgs& a = bs.args;
+        a.G = b->wide ? tile_width(f32, a.n, grouped_lines(a), budget) : 8;
+        a.ngroups = (grouped_lines(a) + a.G - 1) / a.G;
+        const size_t bytes = tile_bytes_of(f32, a.G, a.n);
+        bs.groups = 1;
+        while (b->wide && bs.groups < kBatchWideGroups && 2 * bs.groups * bytes <= budget) bs.groups *= 2;
+        bs.group_elems = (int)(bytes / E);
+        b->smem = std::max(b->smem, bs.groups * bytes);
+    }
     b->ctr_bytes = sizeof(BatchCounters) + sizeof(unsigned) * (size_t)3 * count;
-    const size_t stage_bytes = st.size() * sizeof(StageArgs), plan_bytes = plans.size() * sizeof(MixPlan);
+    const size_t stage_bytes = st.size() * sizeof(BatchStage), plan_bytes = plans.size() * sizeof(MixPlan);
     if (dev_malloc((void**)&b->d_stages, stage_bytes + plan_bytes) ||
         dev_malloc((void**)&b->d_item_base, sizeof(int64_t) * (size_t)(2 * (3 * count + 1))) ||
         dev_malloc((void**)&b->d_need, sizeof(unsigned) * (size_t)(2 * 3 * count)) ||
@@ -194,19 +237,20 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
         return fail(OPENFFT_ERR_NOMEM, "batched plan tables");
     }
     // launch shape: persistent, as many CTAs as fit (tile buffer + queue tables)
-    if (b->smem + tables > 200 * 1024) { free_batch(b); return fail(OPENFFT_ERR_UNSUPPORTED, "batch too large for the queue tables in shared memory"); }
+    if (b->smem + tables > kMaxBatchSmem) { free_batch(b); return fail(OPENFFT_ERR_UNSUPPORTED, "batch too large for the queue tables in shared memory"); }
     // The kernel's shared-memory limit is the same for every plan: plans of other sizes share
     // the kernel, and this one's launches are captured at its first calls.
     int per_sm = 1;
-    e = prepare_kernel(kernel_of(f32, b->G), nullptr);
-    if (!e) e = resident_ctas_per_sm(kernel_of(f32, b->G), kBatchThreads, b->smem + tables, &per_sm);
+    e = prepare_kernel(kernel_of(f32, b->wide), nullptr, (int)kMaxBatchSmem);
+    if (!e) e = resident_ctas_per_sm(kernel_of(f32, b->wide), threads_of(b->wide), b->smem + tables, &per_sm);
     if (e) { free_batch(b); return fail(OPENFFT_ERR_CUDA, cudaGetErrorString(e)); }
     b->grid = sms * (per_sm > 0 ? per_sm : 1);
     {
-        int64_t tiles = 0;                       // of one direction's three stages
-        for (int q = 0; q < 3 * count; ++q) tiles += st[q].ngroups * (st[q].group_i2 ? st[q].M1 : st[q].M2);
-        const int64_t per = tiles / 3 / ((int64_t)b->grid * kItemsPerCta);
-        b->tiles_per_item = (int)(per < 1 ? 1 : (per > kMaxTilesPerItem ? kMaxTilesPerItem : per));
+        int64_t rounds = 0;                      // of one direction's three stages: a tile for each group
+        for (int q = 0; q < 3 * count; ++q) rounds += (tiles_of(st[q].args) + st[q].groups - 1) / st[q].groups;
+        const int64_t per = rounds / 3 / ((int64_t)b->grid * kItemsPerCta);
+        for (BatchStage& bs : st)
+            bs.tiles_per_item = bs.groups * (int)(per < 1 ? 1 : (per > kMaxTilesPerItem ? kMaxTilesPerItem : per));
     }
     // per direction (the two traverse the axes in opposite orders): tiles per
     // (stage, transform) and the stage-major queue prefix
@@ -215,9 +259,8 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
     for (int dir = 0; dir < 2; ++dir) {
         int64_t acc = 0;
         for (int q = 0; q < 3 * count; ++q) {
-            const StageArgs& a = st[(size_t)dir * 3 * count + q];
-            const int64_t tiles = a.ngroups * (a.group_i2 ? a.M1 : a.M2);
-            const int64_t items = (tiles + b->tiles_per_item - 1) / b->tiles_per_item;
+            const BatchStage& bs = st[(size_t)dir * 3 * count + q];
+            const int64_t items = (tiles_of(bs.args) + bs.tiles_per_item - 1) / bs.tiles_per_item;
             bases[(size_t)dir * (3 * count + 1) + q] = acc;
             needs[(size_t)dir * 3 * count + q] = (unsigned)items;
             acc += items;
@@ -228,7 +271,7 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
     // the stage descriptors, then the radix plans they point to
     std::vector<unsigned char> up(stage_bytes + plan_bytes);
     const MixPlan* d_plans = reinterpret_cast<const MixPlan*>(reinterpret_cast<unsigned char*>(b->d_stages) + stage_bytes);
-    for (StageArgs& a : st) a.aux = d_plans + reinterpret_cast<size_t>(a.aux);
+    for (BatchStage& bs : st) bs.args.aux = d_plans + reinterpret_cast<size_t>(bs.args.aux);
     std::memcpy(up.data(), st.data(), stage_bytes);
     std::memcpy(up.data() + stage_bytes, plans.data(), plan_bytes);
     e = cudaMemcpy(b->d_stages, up.data(), up.size(), cudaMemcpyHostToDevice);
@@ -256,7 +299,6 @@ static cudaError_t launch_batch(BatchPlan* b, int dir_index, cudaStream_t s)
     d.ctr = reinterpret_cast<BatchCounters*>(b->d_ctr);
     d.done = reinterpret_cast<unsigned*>(b->d_ctr + sizeof(BatchCounters));
     d.count = b->count;
-    d.tiles_per_item = b->tiles_per_item;
     d.dir_index = dir_index;
     d.wait_budget = b->wait_budget;
     cudaError_t e = cudaMemsetAsync(b->d_ctr, 0, b->ctr_bytes, s);
@@ -266,7 +308,7 @@ static cudaError_t launch_batch(BatchPlan* b, int dir_index, cudaStream_t s)
     const size_t tables = sizeof(int64_t) * (size_t)(3 * b->count + 1) + sizeof(unsigned) * (size_t)(3 * b->count);
     const size_t sm = b->smem + tables;
     void* args[] = {&d, &b->smem};
-    return cudaLaunchKernel(kernel_of(b->arith == ARITH_F32, b->G), dim3((unsigned)b->grid), dim3(kBatchThreads), args, sm, s);
+    return cudaLaunchKernel(kernel_of(b->arith == ARITH_F32, b->wide), dim3((unsigned)b->grid), dim3(threads_of(b->wide)), args, sm, s);
 }
 
 int batch_exec(BatchPlan* b, const void* const* in, void* const* out, int dir, cudaStream_t user,

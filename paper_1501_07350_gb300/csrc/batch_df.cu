@@ -1,16 +1,12 @@
-// batch_df.cu -- the batched kernel in packed double-float.
+// batch_df.cu -- the batched kernels in packed double-float.
 #include "batch_kernel.cuh"
 
 namespace ofg {
 
-size_t batch_tile_bytes_df(int G, int n)
+size_t batch_tile_bytes_df(int G, int n) { return batch_tile_bytes<ArDP>(G, n); }
+const void* batch_kernel_df(bool wide)
 {
-    return G == 8 ? batch_tile_bytes<ArDP, 8>(n) : (G == 4 ? batch_tile_bytes<ArDP, 4>(n) : batch_tile_bytes<ArDP, 2>(n));
-}
-const void* batch_kernel_df(int G)
-{
-    return G == 8 ? (const void*)batch_kernel<ArDP, 8>
-                  : (G == 4 ? (const void*)batch_kernel<ArDP, 4> : (const void*)batch_kernel<ArDP, 2>);
+    return wide ? (const void*)batch_kernel<ArDP, true> : (const void*)batch_kernel<ArDP, false>;
 }
 
 }  // namespace ofg

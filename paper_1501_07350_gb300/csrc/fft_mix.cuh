@@ -70,21 +70,25 @@ __device__ __forceinline__ ArDP::C c128_bits(ArDP::C x)
     return Io<ArDP>::from_c128(make_double2(__longlong_as_double((long long)x.x), __longlong_as_double((long long)x.y)));
 }
 
+// Tiles of G lines (G = 0: a width w that is given at run time).
 template <class A, int G>
 struct Mix {
     using C = typename A::C;
     static constexpr int E = sizeof(C);
     // lanes of a warp: lines fastest, or (line, slot parity) with the parity fastest
-    static constexpr bool kPairs = E * G != 128 || E == 8;
+    __host__ __device__ static constexpr bool pairs(int w) { return E * w != 128 || E == 8; }
     static constexpr int kUnits = 128 / E;                    // elements of one shared-memory wavefront
 
-    __host__ __device__ static int pitch(int n)
+    __host__ __device__ static int pitch(int n, int w = G)
     {
-        if (!kPairs) return n | 1;
+        if (!pairs(w)) return n | 1;
         return n + (2 - n % kUnits + kUnits) % kUnits;
     }
-    __device__ __forceinline__ static int line_of(int tid) { return kPairs ? (tid >> 1) % G : tid % G; }
-    __device__ __forceinline__ static int slot_of(int tid) { return kPairs ? (tid & 1) + 2 * (tid / (2 * G)) : tid / G; }
+    __device__ __forceinline__ static int line_of(int tid, int w = G) { return pairs(w) ? (tid >> 1) % w : tid % w; }
+    __device__ __forceinline__ static int slot_of(int tid, int w = G)
+    {
+        return pairs(w) ? (tid & 1) + 2 * (tid / (2 * w)) : tid / w;
+    }
 
     // Copies of a tile: `valid` lines, lstride apart from line0 on, a warp per line
     // in 16-byte pieces (8 bytes where an odd length or the array's address leaves
@@ -213,38 +217,50 @@ struct Mix {
     }
 };
 
-// Tiles tile, tile + step, ... below end of a stage, by a CTA of T threads.  cur and
-// oth: two tile buffers of G ld elements; tw: n elements for the length's twiddle
-// table, copied in here.  rows: the last pass, whose lines go out as they are, takes
-// consecutive threads along a line.  Returns with the CTA's threads still reading the
-// buffers.
-template <class A, int G, bool REPEAT>
+// Barrier of the threads that run a tile: the CTA's, or that of a group of its warps.
+struct CtaSync {
+    __device__ __forceinline__ void operator()() const { __syncthreads(); }
+};
+struct GroupSync {
+    int id, threads;
+    __device__ __forceinline__ void operator()() const
+    {
+        asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+    }
+};
+
+// Tiles tile, tile + step, ... below end of a stage, by T threads (tid among them) that
+// `sync` synchronises.  cur and oth: two tile buffers of G ld elements; tw: n elements
+// for the length's twiddle table, copied in here.  rows: the last pass, whose lines go
+// out as they are, takes consecutive threads along a line.  Returns with the threads
+// still reading the buffers.
+template <class A, int G, bool REPEAT, class Sync>
 __device__ __forceinline__ void mix_run(const StageArgs& p, const MixPlan& plan, int64_t tile, int64_t step, int64_t end,
-                                        typename A::C* cur, typename A::C* oth, typename A::C* tw, int ld, int slots, int T,
-                                        bool rows)
+                                        typename A::C* cur, typename A::C* oth, typename A::C* tw, int ld, int slots, int tid,
+                                        int T, bool rows, Sync sync)
 {
     using M = Mix<A, G>;
     using C = typename A::C;
-    const int tid = threadIdx.x;
-    const int g = M::line_of(tid), slot = M::slot_of(tid), at = g * ld;
+    const int w = G ? G : p.G;
+    const int g = M::line_of(tid, w), slot = M::slot_of(tid, w), at = g * ld;
     const int gl = rows ? tid / slots : g, sl = rows ? tid - gl * slots : slot, al = gl * ld;      // of the last pass
-    TileGeom tg = tile_geom<REPEAT>(p, tile, G);
+    TileGeom tg = tile_geom<REPEAT>(p, tile, w);
     for (int i = tid; i < p.n; i += T) cp_async<M::E>(tw + i, reinterpret_cast<const C*>(p.tw) + i);
     M::issue_load(p, tg.line0, tg.lstride, tg.valid, cur, ld, tid, T);
     for (; tile < end; tile += step) {
         const int64_t next = tile + step;
-        const TileGeom tn = tile_geom<REPEAT>(p, next < end ? next : tile, G);
+        const TileGeom tn = tile_geom<REPEAT>(p, next < end ? next : tile, w);
         const bool mine = g < tg.valid;
         cp_async_wait_all();
-        __syncthreads();
+        sync();
         const int np = plan.npass;
         if (np > 1) {
             if (mine) M::template dispatch<true>(p, plan.pass[0], false, tg, cur + at, oth + at, tw, g, slot, slots);
-            __syncthreads();
+            sync();
             for (int ps = 1; ps < np - 1; ++ps) {
                 C* t = cur; cur = oth; oth = t;
                 if (mine) M::template dispatch<false>(p, plan.pass[ps], false, tg, cur + at, oth + at, tw, g, slot, slots);
-                __syncthreads();
+                sync();
             }
             // every thread has read `cur`: it takes the next tile while the last pass runs
             if (next < end) M::issue_load(p, tn.line0, tn.lstride, tn.valid, cur, ld, tid, T);
@@ -270,7 +286,7 @@ fft_mix_kernel(const StageArgs p, const __grid_constant__ MixPlan plan, int64_t 
     grid_wait();
     // the grid has at most ntiles CTAs
     mix_run<A, G, REPEAT>(p, plan, blockIdx.x, gridDim.x, ntiles, buf, buf + G * ld, buf + 2 * G * ld, ld, plan.slots,
-                          blockDim.x, sizeof(C) == 8 && rows);
+                          threadIdx.x, blockDim.x, sizeof(C) == 8 && rows, CtaSync());
 }
 
 // The radix plan of length n for a policy of 16-byte (double-float) or 8-byte (FP32)

@@ -66,10 +66,10 @@ const MixLaunch& mix_launch(int n)
 }
 
 // A kernel's dynamic shared-memory limit and carveout, set once per device.
-inline cudaError_t prepare_kernel(const void* kern, int* slot)
+inline cudaError_t prepare_kernel(const void* kern, int* slot, int max_smem = 200 * 1024)
 {
     if (slot && *slot) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
     if (!e) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (!e && slot) *slot = 1;
     return e;

@@ -150,3 +150,71 @@ def test_plans_of_several_sizes_at_once(torch, dtype, tol):
     finally:
         for plan in plans:
             of.openfft_destroy(plan)
+
+
+# The kernel of plans with a long axis: tiles of 8, 4, 2 and 1 lines, one, two and four
+# groups of threads, fewer tiles than groups, ragged last tiles, fewer lines than a tile.
+@pytest.mark.parametrize("dtype,tol", [(of.C2C_F32, 1e-5), (of.C2C_F64, 1e-12)])
+@pytest.mark.parametrize("shapes", [[(2048, 9, 5), (30, 36, 40)], [(600, 7, 9), (300, 5, 4), (48, 10, 9), (2, 3, 1)],
+                                    [(1, 1792, 6), (375, 3, 30), (360, 7, 2)], [(1024, 10, 3), (21, 500, 1), (1, 1, 700)],
+                                    [(96, 1250, 2), (7, 9, 10)] + [(16, 18, 20)] * 30])
+def test_long_axes_beside_short_ones(torch, shapes, dtype, tol):
+    Ps = [1] * len(shapes)
+    plan = of.openfft_plan_many(shapes, Ps, dtype)
+    try:
+        xs, xd = _inputs(torch, shapes, 51, dtype)
+        _check_batch(torch, plan, shapes, Ps, xs, xd, dtype, tol)
+    finally:
+        of.openfft_destroy(plan)
+
+
+@pytest.mark.parametrize("dtype", [of.C2C_F32, of.C2C_F64])
+def test_a_long_axis_does_not_slow_the_others(torch, dtype):
+    """One 2048x48x48 beside 63 48^3 takes no longer than the two as batches of their own
+    (and a third of that)."""
+    tdt = torch.complex64 if dtype == of.C2C_F32 else torch.complex128
+
+    def best(shapes):
+        plan = of.openfft_plan_many(shapes, [1] * len(shapes), dtype)
+        try:
+            of.openfft_set_stream(plan, torch.cuda.current_stream())
+            xs = [torch.randn(int(np.prod(s)), device="cuda", dtype=tdt) for s in shapes]
+            ys = [torch.empty_like(x) for x in xs]
+            times = []
+            for _ in range(12):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                of.openfft_exec_many(plan, xs, ys, of.FORWARD)
+                b.record()
+                of.openfft_sync(plan)
+                torch.cuda.synchronize()
+                times.append(a.elapsed_time(b))
+            return min(times)
+        finally:
+            of.openfft_destroy(plan)
+
+    long, short = [(2048, 48, 48)], [(48, 48, 48)] * 63
+    assert best(long + short) < 4 / 3 * (best(long) + best(short))
+
+
+@pytest.mark.parametrize("shape,count,dtype", [((1, 1, 1), 5687, of.C2C_F32), ((3, 3, 3), 5666, of.C2C_F32),
+                                               ((1, 1, 1), 5686, of.C2C_F64), ((2048, 1, 1), 3868, of.C2C_F32),
+                                               ((2048, 1, 1), 2047, of.C2C_F64)])
+def test_the_largest_counts(torch, shape, count, dtype):
+    """As many transforms as the queue tables leave room for beside the narrowest tiles."""
+    tdt = torch.complex64 if dtype == of.C2C_F32 else torch.complex128
+    n = int(np.prod(shape))
+    plan = of.openfft_plan_many([shape] * count, [1] * count, dtype)
+    try:
+        of.openfft_set_stream(plan, torch.cuda.current_stream())
+        x = torch.randn((count, n), device="cuda", dtype=tdt)
+        y = torch.full_like(x, float("nan"))
+        of.openfft_exec_many(plan, list(x), list(y), of.FORWARD)
+        of.openfft_sync(plan)
+        want = torch.fft.fftn(x.to(torch.complex128).reshape((count,) + shape), dim=(1, 2, 3)).permute(0, 3, 2, 1).reshape(count, n)
+        assert float(torch.linalg.vector_norm(y - want) / torch.linalg.vector_norm(want)) < (1e-5 if dtype == of.C2C_F32 else 1e-12)
+    finally:
+        of.openfft_destroy(plan)
+    with pytest.raises(of.OpenFFTError) as ei:
+        of.openfft_plan_many([shape] * 6000, [1] * 6000, dtype)
+    assert ei.value.status == of.ERR_UNSUPPORTED
