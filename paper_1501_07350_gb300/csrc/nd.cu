@@ -145,7 +145,7 @@ int add_stage(openfft_nd_plan_s* p, std::vector<NdLaunch>& ops, int axis, int64_
     a.conj_out = (dir == OPENFFT_BACKWARD && last) ? 1 : 0;
     a.scale = a.conj_out ? 1.0 / (double)p->N : 1.0;
     L.arith = p->arith;
-    L.grid = a.ngroups * (group_i2 ? M1 : M2) * M3;
+    L.grid = a.ngroups * (group_i2 ? M1 : M2);      // of one i3: a geometry too large for one launch has one per i3
     L.smem = 2 * (size_t)n * (G + 1) * E;
     L.sms = p->sms;
     L.family = KERNEL_AUTO;

@@ -123,3 +123,10 @@ def test_repeated_line_geometry(torch, dims, dtype):
             assert oracle.rel_l2(yd.cpu().numpy().astype(np.complex128), ref) < tol, (dims, direction)
     finally:
         of.openfft_nd_destroy(plan)
+
+
+def test_more_tiles_than_one_launch_takes(torch):
+    """Stages whose repeated geometry has 2^31 tiles or more have a launch per block: the
+    plan is made (2^31 points of complex64, 17 GB of workspace)."""
+    plan = of.openfft_nd_plan((2048, 1024, 1, 1, 1024), 1, of.C2C_F32)
+    of.openfft_nd_destroy(plan)
