@@ -2,6 +2,7 @@
 #pragma once
 #include <algorithm>
 #include <atomic>
+#include <new>
 
 #include "fft_mix.cuh"
 
@@ -46,20 +47,21 @@ MixLaunch make_launch(int n)
 }
 
 // The launch of length n that `make` makes, made on its first use and kept in `made`
-// (kMaxLen + 1 entries); two threads may both make one, and one is kept.
+// (kMaxLen + 1 entries); two threads may both make one, and one is kept.  Without host
+// memory to keep it in, it is made again at the next call.
 template <class Make>
-const MixLaunch& kept_launch(std::atomic<const MixLaunch*>* made, int n, Make make)
+MixLaunch kept_launch(std::atomic<const MixLaunch*>* made, int n, Make make)
 {
-    const MixLaunch* l = made[n].load(std::memory_order_acquire);
-    if (l) return *l;
-    const MixLaunch* mine = new MixLaunch(make(n));
-    if (made[n].compare_exchange_strong(l, mine, std::memory_order_acq_rel)) return *mine;
-    delete mine;
-    return *l;
+    const MixLaunch* kept = made[n].load(std::memory_order_acquire);
+    if (kept) return *kept;
+    const MixLaunch l = make(n);
+    const MixLaunch* mine = new (std::nothrow) MixLaunch(l);
+    if (mine && !made[n].compare_exchange_strong(kept, mine, std::memory_order_acq_rel)) delete mine;
+    return l;
 }
 
 template <class A, int G>
-const MixLaunch& mix_launch(int n)
+MixLaunch mix_launch(int n)
 {
     static std::atomic<const MixLaunch*> made[kMaxLen + 1] = {};
     return kept_launch(made, n, make_launch<A, G>);
@@ -78,7 +80,7 @@ inline cudaError_t prepare_kernel(const void* kern, int* slot, int max_smem = 20
 template <class A, int G, bool REPEAT>
 cudaError_t launch_mix_r(const StageLaunch& L, cudaStream_t st, bool* handled)
 {
-    const MixLaunch& ml = mix_launch<A, G>(L.args.n);
+    const MixLaunch ml = mix_launch<A, G>(L.args.n);
     if (ml.plan.npass == 0) return cudaSuccess;
     auto kern = fft_mix_kernel<A, G, REPEAT>;
     static int cached[kMaxDevices] = {};          // 1 once the kernel's attributes are set on the device

@@ -2,7 +2,6 @@
 #include "fft_mix.cuh"
 
 #include <iterator>
-#include <vector>
 
 namespace ofg {
 
@@ -20,19 +19,31 @@ constexpr int kRadixF32[] = {16, 15, 12, 10, 9, 8, 7, 6, 5, 4, 3, 2};
 // points and 1.5 up to 64, where more threads with less to do each win: 48^3 took
 // 12.1 us as 4 4 3, 15.1 as 8 6; 80^3 29 as 5 4 4, 36 as 10 8; 144^3 110 as 8 6 3, 115
 // as 4 4 3 3.
-void mix_search(const int* radix, int count, int rest, float pass, std::vector<int>& cur, std::vector<int>& best)
+// Plans are made in the calls that execute transforms: no container, nothing that throws.
+struct Radices {
+    int r[kMixMaxPasses];
+    int count = 0;
+    float cost(float pass) const
+    {
+        float c = pass * count;
+        for (int i = 0; i < count; ++i) c += r[i];
+        return c;
+    }
+};
+
+void mix_search(const int* radix, int kinds, int rest, float pass, Radices& cur, Radices& best)
 {
     if (rest == 1) {
-        auto cost = [pass](const std::vector<int>& v) { float s = pass * v.size(); for (int r : v) s += r; return s; };
-        if (best.empty() || cost(cur) < cost(best)) best = cur;
+        if (best.count == 0 || cur.cost(pass) < best.cost(pass)) best = cur;
         return;
     }
-    for (int i = 0; i < count; ++i) {
+    if (cur.count == kMixMaxPasses) return;
+    for (int i = 0; i < kinds; ++i) {
         const int R = radix[i];
-        if (rest % R || (!cur.empty() && R > cur.back())) continue;
-        cur.push_back(R);
-        mix_search(radix, count, rest / R, pass, cur, best);
-        cur.pop_back();
+        if (rest % R || (cur.count && R > cur.r[cur.count - 1])) continue;
+        cur.r[cur.count++] = R;
+        mix_search(radix, kinds, rest / R, pass, cur, best);
+        --cur.count;
     }
 }
 
@@ -43,13 +54,13 @@ MixPlan mix_radix_plan(int n, bool df)
     MixPlan pl;
     pl.npass = 0;
     pl.slots = 1;
-    std::vector<int> cur, best;
-    if (n == 1) best = {1};
+    Radices cur, best;
+    if (n == 1) best.r[best.count++] = 1;
     else if (df) mix_search(kRadixDF, (int)std::size(kRadixDF), n, n <= 64 ? 1.5f : (n <= 100 ? 3.5f : 6.5f), cur, best);
     else mix_search(kRadixF32, (int)std::size(kRadixF32), n, 100.f, cur, best);
-    if (best.size() > (size_t)kMixMaxPasses) return pl;
     int m = 1;
-    for (int R : best) {
+    for (int i = 0; i < best.count; ++i) {
+        const int R = best.r[i];
         MixPass& ps = pl.pass[pl.npass++];
         ps.radix = R;
         ps.nbf = n / R;

@@ -7,7 +7,7 @@ namespace ofg {
 namespace {
 
 template <class A, int G>
-const MixLaunch& real_launch(int n)
+MixLaunch real_launch(int n)
 {
     static std::atomic<const MixLaunch*> made[kMaxLen + 1] = {};
     return kept_launch(made, n, [](int len) {
@@ -22,7 +22,7 @@ const MixLaunch& real_launch(int n)
 template <class A, int G>
 cudaError_t launch_real_g(const StageLaunch& L, cudaStream_t st, bool* handled)
 {
-    const MixLaunch& ml = real_launch<A, G>(L.args.n);
+    const MixLaunch ml = real_launch<A, G>(L.args.n);
     if (ml.plan.npass == 0) return cudaSuccess;
     const bool fwd = L.family == KERNEL_R2C;
     static int cached[2][kMaxDevices] = {};
