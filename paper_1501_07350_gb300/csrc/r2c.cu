@@ -19,8 +19,8 @@
 // Power-of-two n (32..512): one warp per complex line (a pair of real lines)
 // in the padded per-warp layout of the warp-per-line stage kernel, with its
 // radix passes; persistent CTAs of 8 warps.  Other n: the any-length kernel
-// (r2c_mix.cuh); on small arrays, where its tiles do not fit shared memory (about 1000
-// points) and for native FP64, one CTA per tile of 2G real lines (G complex lines) in
+// (r2c_mix.cuh); on small arrays and long ones of lines of a few points, where its tiles
+// do not fit shared memory (about 1000 points) and for native FP64, one CTA per tile of 2G real lines (G complex lines) in
 // two ping-pong [n][G + 1] shared-memory tiles, with the radix passes of the generic
 // stage kernel (any supported n, runtime radix plan).
 #include <cuda_runtime.h>
@@ -499,7 +499,18 @@ cudaError_t launch_real_stage(const StageLaunch& L, cudaStream_t st)
     // 637 -> 558).  The warp kernels are faster on the other powers of two (256^3 258 against
     // 289, inverse 248 against 280; in float 97 against 99, inverse 95 against 117).
     const int n = L.args.n;
-    const bool any = warp_length(n) ? L.arith == ARITH_DF && (n == 128 || n == 512) : L.args.M1 * n >= 32768;
+    const int64_t lines = L.args.M1;
+    bool any = warp_length(n) ? L.arith == ARITH_DF && (n == 128 || n == 512) : lines * n >= 32768;
+    // Its tile of 16 lines is only a few hundred bytes on lines of a few points, and a long
+    // array of those waits at its barriers.  Lines of one point stay on the generic stage from
+    // 2^18 lines in FP32 (2^21 lines 124 us against 219, inverse 163 against 291) and in the
+    // double-float inverse from 2^17 (449 against 535; forward 445 against 269).  So do those
+    // of the FP32 inverse beyond 2^20 lines where the generic stage has one pass (2^21 lines
+    // of 2 points 290 us against 336, of 5 381 against 405, of 7 420 against 436; of 6, two
+    // passes, 471 against 427; 2^20 lines of 2 points 154 and 155, of 7 216 and 197).
+    const bool f32 = L.arith == ARITH_F32, inverse = L.family == KERNEL_C2R;
+    if (n == 1 && (f32 ? lines >= 1 << 18 : inverse && lines >= 1 << 17)) any = false;
+    if (f32 && inverse && n <= 7 && n != 6 && lines > 1 << 20) any = false;
     if (any) {
         bool handled = false;
         cudaError_t e = launch_real_mix(L, st, &handled);

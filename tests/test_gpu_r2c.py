@@ -198,3 +198,56 @@ def test_any_length_real_stages(torch, n, dtype):
         assert oracle.rel_l2(zd.cpu().numpy().astype(np.float64), x.reshape(-1)) < 2 * tol, n
     finally:
         of.openfft_destroy(plan)
+
+
+# Long arrays of lines of a few points, on either side of the counts from which the
+# generic stage takes them: 2^17 and 2^18 lines of one point, 2^20 of two to seven.
+@pytest.mark.parametrize("dtype", [of.R2C_F64, of.R2C_F32])
+@pytest.mark.parametrize("shape", [(256, 500, 1), (256, 512, 1), (512, 500, 1), (512, 512, 1), (1024, 1024, 2), (1024, 1029, 3),
+                                   (1024, 1029, 5), (1029, 1024, 6), (1024, 1029, 7)])
+def test_long_arrays_of_short_lines(torch, shape, dtype):
+    rt, ct = _types(torch, dtype)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn(shape, generator=gen, device="cuda", dtype=rt)
+    want = torch.fft.rfftn(x.to(torch.float64)).permute(2, 1, 0).contiguous().reshape(-1)
+    plan = of.openfft_plan(*shape, 1, dtype)
+    try:
+        of.openfft_set_stream(plan, torch.cuda.current_stream())
+        y = torch.full((want.numel(),), float("nan"), dtype=ct, device="cuda")
+        z = torch.full((x.numel(),), float("nan"), dtype=rt, device="cuda")
+        of.openfft_exec_r2c(plan, x.reshape(-1), y)
+        of.openfft_exec_c2r(plan, want.to(ct), z)
+        of.openfft_sync(plan)
+        assert float(torch.linalg.vector_norm(y - want) / torch.linalg.vector_norm(want)) < TOL[dtype]
+        assert float(torch.linalg.vector_norm(z - x.reshape(-1)) / torch.linalg.vector_norm(x)) < TOL[dtype]
+    finally:
+        of.openfft_destroy(plan)
+
+
+def test_short_lines_do_not_slow_the_inverse(torch):
+    """2^21 real lines of one point: the inverse, which moves less than the complex one
+    and shares its other stages, takes no longer."""
+    shape = (2048, 1024, 1)
+    n = 2048 * 1024
+    rp, cp = of.openfft_plan(*shape, 1, of.R2C_F32), of.openfft_plan(*shape, 1, of.C2C_F32)
+    try:
+        h = torch.randn(n, device="cuda", dtype=torch.complex64)
+        y, z = torch.empty(n, device="cuda"), torch.empty_like(h)
+
+        def best(call):
+            times = []
+            for _ in range(12):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                call()
+                b.record()
+                torch.cuda.synchronize()
+                times.append(a.elapsed_time(b))
+            return min(times)
+
+        for p in (rp, cp):
+            of.openfft_set_stream(p, torch.cuda.current_stream())
+        assert best(lambda: of.openfft_exec_c2r(rp, h, y)) < best(lambda: of.openfft_exec_c2c(cp, h, z, of.BACKWARD))
+    finally:
+        of.openfft_destroy(rp)
+        of.openfft_destroy(cp)
