@@ -503,13 +503,14 @@ cudaError_t launch_real_stage(const StageLaunch& L, cudaStream_t st)
     bool any = warp_length(n) ? L.arith == ARITH_DF && (n == 128 || n == 512) : lines * n >= 32768;
     // Its tile of 16 lines is only a few hundred bytes on lines of a few points, and a long
     // array of those waits at its barriers.  Lines of one point stay on the generic stage from
-    // 2^18 lines in FP32 (2^21 lines 124 us against 219, inverse 163 against 291) and in the
-    // double-float inverse from 2^17 (449 against 535; forward 445 against 269).  So do those
+    // 2^17 lines in FP32 (2^21 lines 124 us against 219, inverse 163 against 291; 2^17 16.4 and
+    // 22.9, inverse 21.2 and 28.5; 102400 alike) and in the double-float inverse (449 against
+    // 535, 38.8 and 47.5; forward 445 against 269).  So do those
     // of the FP32 inverse beyond 2^20 lines where the generic stage has one pass (2^21 lines
     // of 2 points 290 us against 336, of 5 381 against 405, of 7 420 against 436; of 6, two
     // passes, 471 against 427; 2^20 lines of 2 points 154 and 155, of 7 216 and 197).
     const bool f32 = L.arith == ARITH_F32, inverse = L.family == KERNEL_C2R;
-    if (n == 1 && (f32 ? lines >= 1 << 18 : inverse && lines >= 1 << 17)) any = false;
+    if (n == 1 && (f32 || inverse) && lines >= 1 << 17) any = false;
     if (f32 && inverse && n <= 7 && n != 6 && lines > 1 << 20) any = false;
     if (any) {
         bool handled = false;

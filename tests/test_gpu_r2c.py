@@ -201,7 +201,7 @@ def test_any_length_real_stages(torch, n, dtype):
 
 
 # Long arrays of lines of a few points, on either side of the counts from which the
-# generic stage takes them: 2^17 and 2^18 lines of one point, 2^20 of two to seven.
+# generic stage takes them: 2^17 lines of one point, 2^20 of two to seven.
 @pytest.mark.parametrize("dtype", [of.R2C_F64, of.R2C_F32])
 @pytest.mark.parametrize("shape", [(256, 500, 1), (256, 512, 1), (512, 500, 1), (512, 512, 1), (1024, 1024, 2), (1024, 1029, 3),
                                    (1024, 1029, 5), (1029, 1024, 6), (1024, 1029, 7)])
