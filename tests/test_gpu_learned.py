@@ -11,6 +11,7 @@ the LEARNED tuning mode, and the regret of the trained cost model.
 - trained without any problem that has a 512-point axis, its picks on the
   512^3 benchmark problems are within 5 % of exhaustive tuning too.
 """
+import json
 import os
 
 import numpy as np
@@ -128,3 +129,16 @@ def test_trained_model_regret_on_held_out_problems(lib):
             of.openfft_destroy(h)
     finally:
         of.openfft_set_cost_model(0, 0, None)
+
+
+def test_committed_model_on_fresh_timings(lib):
+    """The committed model's picks against exhaustive timings taken now: a model of kernels
+    that have since changed fails here, however well it fits its own dataset."""
+    with open(learned.MODEL_FILE) as fh:
+        model = json.load(fh)
+    params = [np.asarray(p, dtype=np.float32) for p in model["params"]]
+    problems = [((60, 90, 150), 15, "f64"), ((200, 100, 50), 10, "f64"), ((200, 100, 50), 10, "f32"), ((24, 250, 30), 6, "f32"),
+                ((320, 160, 64), 40, "f32"), ((80, 80, 80), 5, "f32"), ((120, 144, 160), 32, "f64"), ((256, 256, 256), 64, "f64")]
+    ev = learned.evaluate(learned.collect(problems), params, model["hidden"])
+    s = learned.summary(ev)
+    assert s["mean_regret"] <= 0.05 and s["max_regret"] <= 0.2, [(e["shape"], e["dtype"], e["pick"], e["regret"]) for e in ev]
