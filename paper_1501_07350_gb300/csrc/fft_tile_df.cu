@@ -16,11 +16,10 @@ cudaError_t launch_tile_df(const StageLaunch& L, cudaStream_t st, bool* handled)
         if (*handled || e) return e;
     }
     // a tile of the warp kernel is one warp of 32-point lines, two of 64-point ones: with
-    // few lines it leaves the chip nearly empty, and fft_mix's tiles are faster (32^3 10.5
-    // against 11.8 us; with 64-point lines on it too, 64x32x32 10.9 against 12.8, 32x32x64
-    // 10.5 against 12.2, 64x64x32 11.8 against 13.3).  Above, the warp kernel: 64^3, 4096
-    // lines, 13.5 against 15.2, 32x32x256, 8192 of 32 points, 14.5 against 16.0, 128x128x32
-    // 21.5 against 25.4.
+    // few lines it leaves the chip nearly empty, and fft_mix's tiles are faster (32^3 10.1
+    // against 11.1 us, 64x32x32 11.4 against 12.2, 32x32x64 10.8 against 12.2, 64x64x32 12.3
+    // against 12.8).  Above, the warp kernel: 64^3, 4096 lines, 13.6 against 15.2, 32x32x256,
+    // 8192 of 32 points, 14.7 against 16.3, 128x128x32 21.7 against 25.6.
     const int64_t lines = choice_lines(L);
     if (L.family == KERNEL_AUTO && ((L.args.n == 32 && lines <= 4096) || (L.args.n == 64 && lines <= 2048))) {
         cudaError_t e = launch_mix_df(L, st, handled);

@@ -8,11 +8,11 @@ namespace ofg {
 cudaError_t launch_tile_f32(const StageLaunch& L, cudaStream_t st, bool* handled)
 {
     *handled = false;
-    // fft_mix also beats the warp kernel on the longer power-of-two lengths (256^3 156
-    // against 172-198 us, 512^3 1460 against 1590-1650) and on 64 and 128 points where
-    // there are lines enough to fill the chip several times (512x64x512 183 against
-    // 194, 512x128x512 354 against 362; 128^3, 16384 lines, 24.0 against 25.7).  64^3 (4096
-    // lines) takes 10.0 against 7.4 us, 128x128x64 (8192 to 16384) 14.5 against 14.0.
+    // fft_mix also takes the longer power-of-two lengths (with the warp kernel 256^3 took
+    // 172-198 us and 512^3 1590-1650, with fft_mix then 156 and 1460), and 64 and 128 points
+    // where there are lines enough to fill the chip several times (512x64x512 161 against
+    // 173, 512x128x512 310 against 321; 128^3, 16384 lines, 24.3 against 25.3).  64^3 (4096
+    // lines) takes 10.1 against 7.3 us, 128x128x64 (8192 to 16384) 14.7 against 14.2.
     const int64_t lines = choice_lines(L);
     if (L.family == KERNEL_AUTO && (L.args.n >= 256 || (L.args.n == 64 && lines >= 32768) || (L.args.n == 128 && lines >= 16384))) {
         cudaError_t e = launch_mix_f32(L, st, handled);

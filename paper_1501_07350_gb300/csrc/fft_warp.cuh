@@ -313,7 +313,8 @@ cudaError_t launch_warp_n(const StageLaunch& L, cudaStream_t st)
     return launch_chained(L, fft_warp_kernel<A, N, G>, (unsigned)grid, T, smem, st, L.args, ntiles);
 }
 
-// power-of-two lengths go to the warp-per-line kernel
+// power-of-two lengths go to the warp-per-line kernel; FP32 lines of 256 points and more
+// have none (fft_mix.cuh takes them all)
 template <class A, int G>
 cudaError_t launch_warp_g(const StageLaunch& L, cudaStream_t st, bool* handled)
 {
@@ -324,10 +325,14 @@ cudaError_t launch_warp_g(const StageLaunch& L, cudaStream_t st, bool* handled)
     case 32: return launch_warp_n<A, 32, G>(L, st);
     case 64: return launch_warp_n<A, 64, G>(L, st);
     case 128: return launch_warp_n<A, 128, G>(L, st);
-    case 256: return launch_warp_n<A, 256, G>(L, st);
-    case 512: return launch_warp_n<A, 512, G>(L, st);
-    default: *handled = false; return cudaSuccess;
+    default: break;
     }
+    if constexpr (sizeof(typename A::C) >= 16) {
+        if (a.n == 256) return launch_warp_n<A, 256, G>(L, st);
+        if (a.n == 512) return launch_warp_n<A, 512, G>(L, st);
+    }
+    *handled = false;
+    return cudaSuccess;
 }
 
 }  // namespace ofg

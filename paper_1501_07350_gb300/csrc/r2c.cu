@@ -25,6 +25,8 @@
 // stage kernel (any supported n, runtime radix plan).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "fft_stage.h"
 #include "fft_warp.cuh"
 #include "generic_stage.cuh"
@@ -458,10 +460,12 @@ cudaError_t launch_real_a(const StageLaunch& L, cudaStream_t st)
     switch (L.args.n) {
     case 32: return launch_real_warp<AW, 32>(L, st);
     case 64: return launch_real_warp<AW, 64>(L, st);
-    case 128: return launch_real_warp<AW, 128>(L, st);
     case 256: return launch_real_warp<AW, 256>(L, st);
-    case 512: return launch_real_warp<AW, 512>(L, st);
     default: break;
+    }
+    if constexpr (!std::is_same<AW, ArDP>::value) {       // double-float lines of 128 and 512 points: launch_real_mix
+        if (L.args.n == 128) return launch_real_warp<AW, 128>(L, st);
+        if (L.args.n == 512) return launch_real_warp<AW, 512>(L, st);
     }
     static int attr_r2c[kMaxDevices] = {}, attr_c2r[kMaxDevices] = {};     // attribute set on that device
     const unsigned grid = (unsigned)L.grid;
@@ -495,9 +499,10 @@ cudaError_t launch_real_stage(const StageLaunch& L, cudaStream_t st)
     // us, inverse 341 -> 315, float 111 -> 85, inverse 112 -> 89; 65536 lines of 9 points in
     // double 38 -> 22, inverse 43 -> 39; 45^3 alike; on a smaller array its few CTAs take
     // longer to a tile: 15^3 in float 10.2 against 13.9) and, in double-float, 128 (128^3
-    // 50.2 -> 47.3, inverse 51.4 -> 46.2) and 512 points (256x256x512 615 -> 559, inverse
-    // 637 -> 558).  The warp kernels are faster on the other powers of two (256^3 258 against
-    // 289, inverse 248 against 280; in float 97 against 99, inverse 95 against 117).
+    // 41.6 against 42.8 with the warp kernel, inverse 42.6 against 44.9) and 512 points
+    // (256x256x512 510 against 523, inverse 504 against 561).  The warp kernels are faster on
+    // the other powers of two (256^3 220 against 266, inverse 209 against 238; in float 83.1
+    // against 85.6, inverse 89.4 against 97.5; 64^3 in float 6.8 against 10.7).
     const int n = L.args.n;
     const int64_t lines = L.args.M1;
     bool any = warp_length(n) ? L.arith == ARITH_DF && (n == 128 || n == 512) : lines * n >= 32768;
