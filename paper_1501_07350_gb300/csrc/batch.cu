@@ -201,6 +201,8 @@ int batch_create(int count, const int* dims, const int* P, int dtype, int sms, B
                 a.group_i2 = g.g2; a.contig_store = g.contig;
                 a.conj_in = g.cin; a.conj_out = g.cout; a.do_fft = 1;
                 a.in_fmt = g.in_fmt; a.out_fmt = g.out_fmt;
+                a.in_elems = a.out_elems = N;          // read by the checked build
+                a.chk = fallback_status_word();
             }
     }
     // Kernel and tile widths.  CTAs of 128 threads and tiles of 8 lines for every stage, while

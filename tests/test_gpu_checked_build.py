@@ -58,3 +58,9 @@ def test_parity_suite_under_the_checked_build(path, expr):
     tail = (r.stdout + r.stderr)[-3000:]
     assert r.returncode == 0, tail
     assert " passed" in r.stdout and " failed" not in r.stdout, tail
+
+
+def test_batched_plans_under_the_checked_build():
+    """The batched kernel runs the stage kernels' checked loads and stores, so its plans have
+    to give the lengths of their arrays."""
+    test_parity_suite_under_the_checked_build("tests/test_gpu_batch.py", "not slow_the_others")
