@@ -257,9 +257,11 @@ int openfft_set_tuning(openfft_plan_t plan, int mode, int candidate);
 
 /* Stage-kernel families: one warp per line (power-of-two lengths 32..512),
  * tiles of lines specialised per length, or the generic kernel (any length);
- * AUTO takes the warp kernel where it exists, for the other lengths (and not
- * for NATIVE arithmetic) tiles with a radix plan chosen per length, else the
- * tile or the generic kernel. */
+ * AUTO takes, except for NATIVE arithmetic, tiles with a radix plan chosen per
+ * length, and the warp kernel on the power-of-two lengths where it is faster
+ * (double-float: all but 32 and 64 points on few lines; FP32: 32 points, and 64
+ * and 128 on few lines); NATIVE takes the warp kernel where it exists; what
+ * none of these takes, the tile or the generic kernel. */
 enum { OPENFFT_KERNEL_AUTO = 0, OPENFFT_KERNEL_WARP = 1, OPENFFT_KERNEL_TILE = 2, OPENFFT_KERNEL_GENERIC = 3 };
 
 /* Number of execution candidates of this plan and a description of one

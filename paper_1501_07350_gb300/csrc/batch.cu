@@ -14,8 +14,8 @@
 //
 // Per item the CTA runs the any-length stage computation (fft_mix.cuh) with the
 // length's radix plan.  Data written by one CTA and read by another in a later stage
-// is loaded with cp.async (after an acquire on the counter, and by a launch whose L1
-// holds no older copy of it); writers fence before releasing.
+// is loaded with cp.async after an acquire on the counter (a device-scope fence, which
+// also covers the copies that go through L1); writers fence before releasing.
 //
 // The time is the tiles': small CTAs (128 threads, up to 8 per SM) keep copies, passes
 // and stores of different items in flight.  64 uneven complex64 transforms (48^3 to

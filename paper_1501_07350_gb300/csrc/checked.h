@@ -1,7 +1,7 @@
 // checked.h -- bounds checks of the checked build (-DOPENFFT_CHECKED).
 //
 // In the checked build every global element index of the C2C stage kernels,
-// the explicit transpose kernels and the multi-device pack / unpack kernels
+// the batched kernel, the explicit transpose kernels and the multi-device pack / unpack kernels
 // is tested against the length of the array it addresses before the access.
 // An index outside [0, lim) is not accessed: the thread skips that element,
 // and the first such index found stores OPENFFT_ERR_BOUNDS (9) in a device

@@ -1,6 +1,10 @@
 // fft_mix.cuh -- FFT stage kernel for the line lengths that have no kernel
-// compiled for them alone: any n <= 2048 with factors 2, 3, 5 and 7, in the packed
-// double-float and the FP32 arithmetic.
+// compiled for them alone: any n with factors 2, 3, 5 and 7, in the packed double-float
+// and the FP32 arithmetic.  The passes take every n <= 2048 (the batched form runs them
+// all); as a stage of its own it goes as far as the plan's tile width, which comes from
+// the generic kernel's two tiles of n (G + 1) elements in 200 KB: 8 lines in FP32 up to
+// 1422 points, 4 in double-float up to 1280, and as many lines side by side in the output
+// (five, three).  Longer lines and fewer of them run on the generic stage.
 //
 // A CTA takes tiles of G lines.  The radix plan is chosen on the host per length
 // (mix_radix_plan): few passes of large radices (composite ones up to 10 in
@@ -21,6 +25,11 @@
 // between a pass's reads and writes, the radix cases spilled).  The last pass reads
 // one buffer and writes global memory, so the next tile's copies (cp.async) go into
 // the other buffer while it runs.
+//
+// Registers: 64 a thread everywhere (the bound of 512-thread CTAs).  The double-float
+// instances spill 44 bytes of stores and 96 of loads there, the real ones up to 216 and
+// 212, the batched one 184 and 164; FP32 ones none.  The 512-thread batched kernel has
+// 128 registers and no spills.
 //
 // In double-float the instructions bound it (6.5-8.5 a point and stage, 47-55 % of issue
 // slots) with the barriers between passes; FP32 runs at 75-85 % of the copy bandwidth on

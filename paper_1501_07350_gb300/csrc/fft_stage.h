@@ -78,8 +78,10 @@ struct StageLaunch {
 // runs the first and the last stage range by range, gives openfft_exec_c2c's bits.
 inline int64_t choice_lines(const StageLaunch& L) { return L.stage_lines ? L.stage_lines : L.args.M1 * L.args.M2; }
 
-// stage kernel families: warp-per-line (power-of-two n), tile (specialised n),
-// generic (any n); AUTO takes the first that has an instantiation for (n, G)
+// stage kernel families: warp-per-line (power-of-two n), tile (specialised n), generic
+// (any n).  AUTO takes the any-length kernel (fft_mix.cuh), or on power-of-two lengths the
+// warp kernels where they are faster (fft_tile_df.cu, fft_tile_f32.cu), and what neither
+// takes goes to the tile or the generic kernel
 enum { KERNEL_AUTO = 0, KERNEL_WARP = 1, KERNEL_TILE = 2, KERNEL_GENERIC = 3 };
 // the real stages of the real transform (r2c.cu): the forward stage 1 and the
 // inverse's last stage; M1 = number of real lines, G = complex lines per CTA
@@ -152,7 +154,7 @@ cudaError_t launch_tile_df(const StageLaunch& L, cudaStream_t st, bool* handled)
 // the asynchronous-output double-float kernels (fft_tma_256.cu, fft_tma_512.cu)
 cudaError_t launch_warp_tma_256(const StageLaunch& L, cudaStream_t st, bool* handled);
 cudaError_t launch_warp_tma_512(const StageLaunch& L, cudaStream_t st, bool* handled);
-// any length (fft_mix.cu)
+// any length (fft_mix_df.cu, fft_mix_f32.cu)
 cudaError_t launch_mix_df(const StageLaunch& L, cudaStream_t st, bool* handled);
 cudaError_t launch_mix_f32(const StageLaunch& L, cudaStream_t st, bool* handled);
 cudaError_t launch_stage(const StageLaunch& L, cudaStream_t st);
