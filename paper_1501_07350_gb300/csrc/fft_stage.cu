@@ -53,6 +53,7 @@ fft_stage_kernel(const StageArgs p)
 __global__ void twiddle_kernel(int n, int fmt, void* out)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_wait();
     if (e >= n) return;
     double s, c;
     sincospi((double)(2 * (int64_t)e) / (double)n, &s, &c);
@@ -75,6 +76,7 @@ __global__ void twiddle_kernel(int n, int fmt, void* out)
 __global__ void warp_twiddle_kernel(int n, void* out)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_wait();
     if (e >= wtw_count(n)) return;
     int p = 1;
     while (p + 1 < wplan_len(n) && e >= wtw_offset(n, p + 1)) ++p;
@@ -208,9 +210,13 @@ cudaError_t launch_stage(const StageLaunch& L0, cudaStream_t st)
 
 cudaError_t launch_twiddles(int n, int fmt, void* out, cudaStream_t st)
 {
-    twiddle_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, fmt, out);
-    if (fmt == FMT_DF && warp_length(n)) warp_twiddle_kernel<<<(wtw_count(n) + 255) / 256, 256, 0, st>>>(n, out);
-    return cudaGetLastError();
+    // chained to each other: six of them go ahead of the stages of an allocation-free call
+    // (32^3 complex128 40.1 us a call with plain launches, 30.0 chained)
+    const StageLaunch L = {};
+    cudaError_t e = launch_chained(L, twiddle_kernel, (unsigned)((n + 255) / 256), 256, 0, st, n, fmt, out);
+    if (!e && fmt == FMT_DF && warp_length(n))
+        e = launch_chained(L, warp_twiddle_kernel, (unsigned)((wtw_count(n) + 255) / 256), 256, 0, st, n, out);
+    return e;
 }
 
 }  // namespace ofg
